@@ -98,7 +98,32 @@ int ilog2(int64_t v) {
   return l;
 }
 
-void make_geo(Geo& g, int lgN) {
+// Column tiles of 4 columns (8 of 32 points), mid tiles of one row pair (two
+// of 64 points): at least 256 values, one warp.
+void r8_col(Geo& g) {
+  g.col_r8 = 1;
+  g.lgG = g.lgN2 == 5 ? 3 : 2;
+  g.G = 1 << g.lgG;
+  g.col_tile = g.G << g.lgN2;
+  g.col_ctas = g.N1 >> g.lgG;
+}
+void r8_mid(Geo& g) {
+  g.mid_r8 = 1;
+  g.lgU = g.lgN1 == 6 ? 1 : 0;
+  g.U = 1 << g.lgU;
+  g.tile = (2 * g.U) << g.lgN1;
+  g.mid_ctas = (g.N2 >> 1) >> g.lgU;
+}
+
+// Radix-8 tiles of one row pair / four columns (the fewest that fill a
+// 32-byte sector), 8 values per thread: as many CTAs as the length gives and
+// short stages.  Taken where the whole pass is less than about one wave of
+// such CTAs and its time is the latency of one tile; the 4096-value tiles of
+// the long transforms move fewer bytes through shared memory.
+// `small_tiles` 0: 4096-value tiles at every length (grouped launches).
+constexpr int R8_LG_MIN = 11, R8_LG_MAX = 19;
+
+void make_geo(Geo& g, int lgN, bool small_tiles) {
   g.lgN = lgN;
   g.N = 1 << lgN;
   g.lgN2 = lgN / 2 < 10 ? lgN / 2 : 10;
@@ -120,6 +145,11 @@ void make_geo(Geo& g, int lgN) {
   g.mid_ctas = (g.N2 >> 1) >> g.lgU;
   g.col_tile = 4096;
   g.twod = 0;
+  g.col_r8 = g.mid_r8 = 0;
+  if (small_tiles && lgN >= R8_LG_MIN && lgN <= R8_LG_MAX) {
+    r8_col(g);
+    r8_mid(g);
+  }
 }
 
 // 2D DFT of an N2 x N1 array (2^lgN2 rows of 2^lgN1): the same two passes
@@ -146,6 +176,11 @@ void make_geo2d(Geo& g, int lgN2, int lgN1) {
   g.U = 1 << lgU;
   g.mid_ctas = (g.N2 >> 1) >> lgU;
   g.twod = 1;
+  // radix-8 tiles wherever the axis has a static shape for them (the others
+  // fall back to run-time shapes, whose stages cost more at any image size)
+  g.col_r8 = g.mid_r8 = 0;
+  if (lgN2 >= 5 && lgN2 <= 9 && lgN1 >= (lgN2 == 5 ? 3 : 2)) r8_col(g);
+  if (lgN1 >= 6 && lgN1 <= 10 && lgN2 >= 3) r8_mid(g);
 }
 
 // Geometry invariants the pass kernels rely on (checked for every plan).
@@ -153,7 +188,7 @@ bool geo_ok(const Geo& g) {
   if (g.twod)
     return g.N2 >= 2 && g.N1 >= 2 && g.G >= 2 && g.col_ctas >= 1 && g.mid_ctas >= 1 && g.U >= 1 &&
            2 * g.U <= 64 && (2 * g.U) * g.N1 <= g.tile && (g.G << g.lgN2) <= g.col_tile && g.N1 <= 4096 &&
-           (g.col_tile == 4096 || (g.lgN2 == 12 && g.lgG == 2 && g.col_tile == 16384));
+           (g.col_tile == 4096 || g.col_r8 || (g.lgN2 == 12 && g.lgG == 2 && g.col_tile == 16384));
   return g.N1 >= g.N2 && g.N2 >= 2 && g.G >= 2 && g.col_ctas >= 1 && g.mid_ctas >= 1 &&
          2 * g.U <= 64 && (2 * g.U) * g.N1 <= g.tile && (g.G << g.lgN2) <= 4096;
 }
@@ -238,8 +273,8 @@ cudaError_t make_tables(Geo& g, float2* base, cudaStream_t s) {
   if (e == cudaSuccess) e = launch_twiddle(twl, g.N1, g.N, s);
   if (e == cudaSuccess) e = launch_twiddle(twr, g.N2, 2 * (int64_t)g.N, s);
   if (e == cudaSuccess) e = launch_twiddle(tw1h, g.N1, g.N1, s);
-  if (e == cudaSuccess) e = launch_stage_tw(tws1, g.lgN1, stage_tw_count(g.lgN1), s);
-  if (e == cudaSuccess) e = launch_stage_tw(tws2, g.lgN2, stage_tw_count(g.lgN2), s);
+  if (e == cudaSuccess) e = launch_stage_tw(tws1, g.lgN1, g.mid_r8 ? 3 : 4, s);
+  if (e == cudaSuccess) e = launch_stage_tw(tws2, g.lgN2, g.col_r8 ? 3 : 4, s);
   g.tw1 = tw1;
   g.tw2 = tw2;
   g.twl = twl;
@@ -270,14 +305,16 @@ cs_status latched_status(cs_plan_s* p) {
 }
 
 // One solve chunk: `len` iterations, the last of which computes the check
-// statistics; `final_chunk` drops the forward FFT after the last update.
+// statistics when `stats`; `final_chunk` drops the forward FFT after the last
+// update.
 enum SolveKind { K_ISTA = 1, K_ADMM = 2 };
 
-cudaError_t enqueue_chunk(cs_plan_s* p, SolveKind kind, int len, bool final_chunk, cudaStream_t s) {
+cudaError_t enqueue_chunk(cs_plan_s* p, SolveKind kind, int len, bool final_chunk, bool stats,
+                          cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   for (int it = 0; it < len && e == cudaSuccess; ++it) {
     const bool last = it == len - 1;
-    const int flags = last ? (FL_STATS | FL_WRITE_STATE) : 0;
+    const int flags = last ? (FL_WRITE_STATE | (stats ? FL_STATS : 0)) : 0;
     if (kind == K_ISTA) {
       const Geo& g = p->gi;
       e = launch_mid(MID_FWD, kparams(p, g, 0), s);
@@ -285,29 +322,28 @@ cudaError_t enqueue_chunk(cs_plan_s* p, SolveKind kind, int len, bool final_chun
       if (e == cudaSuccess) e = launch_mid(MID_ADJ, kparams(p, g, 0), s);
       if (e == cudaSuccess)
         e = launch_col((last && final_chunk) ? COL_ISTA_LAST : COL_ISTA, kparams(p, g, flags), s);
-      if (e == cudaSuccess && last) e = launch_finalize(p->partials, g.col_ctas, p->stats, s);
+      if (e == cudaSuccess && last && stats) e = launch_finalize(p->partials, g.col_ctas, p->stats, s);
     } else {
       const Geo& g = p->ga;
       e = launch_mid(MID_ADMM, kparams(p, g, 0), s);
       if (e == cudaSuccess)
         e = launch_col((last && final_chunk) ? COL_ADMM_LAST : COL_ADMM, kparams(p, g, flags), s);
-      if (e == cudaSuccess && last) e = launch_finalize(p->partials, g.col_ctas, p->stats, s);
+      if (e == cudaSuccess && last && stats) e = launch_finalize(p->partials, g.col_ctas, p->stats, s);
     }
   }
   return e;
 }
 
-int chunk_kernels(SolveKind kind, int len) { return (kind == K_ISTA ? 4 : 2) * len + 1; }
-
-cudaError_t run_chunk(cs_plan_s* p, SolveKind kind, int len, bool final_chunk) {
-  p->launches += chunk_kernels(kind, len);
-  if (!p->use_graphs) return enqueue_chunk(p, kind, len, final_chunk, p->stream);
-  const uint64_t key = ((uint64_t)kind << 40) | ((uint64_t)final_chunk << 32) | (uint32_t)len;
+cudaError_t run_chunk(cs_plan_s* p, SolveKind kind, int len, bool final_chunk, bool stats) {
+  p->launches += (kind == K_ISTA ? 4 : 2) * len + (stats ? 1 : 0);
+  if (!p->use_graphs) return enqueue_chunk(p, kind, len, final_chunk, stats, p->stream);
+  const uint64_t key =
+      ((uint64_t)kind << 40) | ((uint64_t)stats << 33) | ((uint64_t)final_chunk << 32) | (uint32_t)len;
   auto it = p->graphs.find(key);
   if (it == p->graphs.end()) {
     cudaError_t e = cudaStreamBeginCapture(p->cap, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
-    cudaError_t e2 = enqueue_chunk(p, kind, len, final_chunk, p->cap);
+    cudaError_t e2 = enqueue_chunk(p, kind, len, final_chunk, stats, p->cap);
     cudaGraph_t graph = nullptr;
     e = cudaStreamEndCapture(p->cap, &graph);
     if (e2 != cudaSuccess || e != cudaSuccess) {
@@ -335,7 +371,9 @@ cudaError_t solve_loop(cs_plan_s* p, SolveKind kind, int iters, int* iters_run, 
   while (done < iters) {
     const int len = (iters - done) < ce ? (iters - done) : ce;
     const bool final_chunk = done + len == iters;
-    cudaError_t e = run_chunk(p, kind, len, final_chunk);
+    // the statistics of a check point are formed where somebody reads them:
+    // by the monitor at every one, else by the caller's record at the last
+    cudaError_t e = run_chunk(p, kind, len, final_chunk, watch || (final_chunk && need_stats));
     if (e != cudaSuccess) return e;
     done += len;
     if (watch && !final_chunk) {
@@ -383,7 +421,7 @@ bool valid_ptr(const void* q) { return q != nullptr && ((uintptr_t)q & 7u) == 0;
 
 namespace {
 cs_status build_plan(cs_plan_t* out, int64_t n0, int64_t n1, int64_t m, const int64_t* rows, const double* c,
-                     void* stream);
+                     void* stream, bool small_tiles);
 }  // namespace
 
 extern "C" {
@@ -408,7 +446,7 @@ cs_status cs_plan(cs_plan_t* out, int64_t n, int64_t m, const int64_t* rows, con
   *out = nullptr;
   if (m < 1 || m > n) return CS_ERR_ARG;
   if (n < 64 || n > (int64_t(1) << 22) || (n & (n - 1)) != 0) return CS_ERR_UNSUPPORTED;
-  return build_plan(out, 0, n, m, rows, c, stream);
+  return build_plan(out, 0, n, m, rows, c, stream, true);
 }
 
 cs_status cs_plan_2d(cs_plan_t* out, int64_t n0, int64_t n1, int64_t m, const int64_t* pix, const double* c2,
@@ -418,7 +456,7 @@ cs_status cs_plan_2d(cs_plan_t* out, int64_t n0, int64_t n1, int64_t m, const in
   if (n0 < 8 || n1 < 16 || n0 > 4096 || n1 > 4096 || (n0 & (n0 - 1)) != 0 || (n1 & (n1 - 1)) != 0)
     return CS_ERR_UNSUPPORTED;
   if (m < 1 || m > n0 * n1) return CS_ERR_ARG;
-  return build_plan(out, n0, n1, m, pix, c2, stream);
+  return build_plan(out, n0, n1, m, pix, c2, stream, true);
 }
 
 }  // extern "C"
@@ -429,7 +467,7 @@ namespace {
 // image (flattened row-major, n = n0 n1): geometry, FP64 spectrum, tables,
 // row masks.
 cs_status build_plan(cs_plan_t* out, int64_t n0, int64_t n1, int64_t m, const int64_t* rows, const double* c,
-                     void* stream) {
+                     void* stream, bool small_tiles) {
   const bool twod = n0 > 0;
   const int64_t n = twod ? n0 * n1 : n1;
   cs_plan_s* p = new (std::nothrow) cs_plan_s();
@@ -444,8 +482,8 @@ cs_status build_plan(cs_plan_t* out, int64_t n0, int64_t n1, int64_t m, const in
     make_geo2d(p->gi, ilog2(n0), ilog2(n1) - 1);
     make_geo2d(p->ga, ilog2(n0), ilog2(n1));
   } else {
-    make_geo(p->gi, lgn - 1);
-    make_geo(p->ga, lgn);
+    make_geo(p->gi, lgn - 1, small_tiles);
+    make_geo(p->ga, lgn, small_tiles);
   }
   if (!geo_ok(p->gi) || !geo_ok(p->ga)) {
     delete p;
@@ -471,7 +509,10 @@ cs_status build_plan(cs_plan_t* out, int64_t n0, int64_t n1, int64_t m, const in
     if (e_ != cudaSuccess) return fail(cuda_status(e_));   \
   } while (0)
 
-  CS_PLAN_TRY(init_pass_kernels());
+  for (const Geo* g : {&p->gi, &p->ga}) {
+    CS_PLAN_TRY(init_col_kernels(*g));
+    CS_PLAN_TRY(init_mid_kernels(*g));
+  }
   CS_PLAN_TRY(cudaStreamCreateWithFlags(&p->cap, cudaStreamNonBlocking));
   CS_PLAN_TRY(cudaEventCreate(&p->ev0));
   CS_PLAN_TRY(cudaEventCreate(&p->ev1));
@@ -945,7 +986,7 @@ cs_status cs_grad(cs_plan_t p, const float* y, float lambda, float tau, int T, i
   for (int sg = 0; sg < S; ++sg) {
     const int L = (sg + 1) * K <= T ? K : T - sg * K;
     CS_TRY(cudaMemcpyAsync(G.ckpt + sg * n, p->xi_t, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
-    CS_TRY(run_chunk(p, K_ISTA, L, sg == S - 1));
+    CS_TRY(run_chunk(p, K_ISTA, L, sg == S - 1, false));
   }
   p->ista_args = false;
   p->admm_args = false;
@@ -1127,7 +1168,7 @@ extern "C" cs_status cs_grad_admm(cs_plan_t p, const float* y, float lambda, con
     const int L = (sg + 1) * K <= T ? K : T - sg * K;
     for (int i = 0; i < 4; ++i)
       CS_TRY(cudaMemcpyAsync(G.ckpt + (sg * 4 + i) * n, state[i], nb, cudaMemcpyDeviceToDevice, s));
-    CS_TRY(run_chunk(p, K_ADMM, L, sg == S - 1));
+    CS_TRY(run_chunk(p, K_ADMM, L, sg == S - 1, false));
   }
 
   // per-iteration arguments: replay (state in the plan's buffers), reverse,
@@ -1198,6 +1239,10 @@ extern "C" cs_status cs_grad_admm(cs_plan_t p, const float* y, float lambda, con
 // ------------------------------------------------------ grouped launches
 
 namespace csk {
+
+int plan_for_group(cs_plan_s** out, int64_t n, int64_t m, const int64_t* rows, const double* c, void* stream) {
+  return build_plan(out, 0, n, m, rows, c, stream, false);
+}
 
 PlanView plan_view(cs_plan_s* p) {
   PlanView v{};

@@ -42,12 +42,12 @@ __global__ void twiddle_k(float2* dst, int count, int64_t M) {
 // Stage-major twiddle table of a length-L FFT (see stage_twiddle): the
 // stage with span Ls and radix R holds w_{Ls R}^(r k) at row(r) Ls + k for
 // the rows r it keeps (tw_row_r).
-__global__ void stage_tw_k(float2* dst, int lgL, int count) {
+__global__ void stage_tw_k(float2* dst, int lgL, int lgRmax, int count) {
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= count) return;
-  int lgLs = 4;
+  int lgLs = lgRmax;
   while (true) {
-    const int lgR = (lgL - lgLs) >= 4 ? 4 : (lgL - lgLs);
+    const int lgR = (lgL - lgLs) >= lgRmax ? lgRmax : (lgL - lgLs);
     const int sz = tw_rows(lgR) << lgLs;
     if (t < sz) {
       const int r = tw_row_r(lgR, t >> lgLs), k = t & ((1 << lgLs) - 1);
@@ -454,8 +454,9 @@ cudaError_t launch_tab_ista(const double2* chat, const Geo& g, int64_t n, float4
   return cudaGetLastError();
 }
 
-cudaError_t launch_stage_tw(float2* dst, int lgL, int count, cudaStream_t s) {
-  if (count > 0) stage_tw_k<<<blocks_for(count), AUX_NT, 0, s>>>(dst, lgL, count);
+cudaError_t launch_stage_tw(float2* dst, int lgL, int lgRmax, cudaStream_t s) {
+  const int count = stage_tw_count(lgL, lgRmax);
+  if (count > 0) stage_tw_k<<<blocks_for(count), AUX_NT, 0, s>>>(dst, lgL, lgRmax, count);
   return cudaGetLastError();
 }
 

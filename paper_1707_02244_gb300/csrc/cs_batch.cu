@@ -608,13 +608,15 @@ cs_status cs_batch_plan(cs_batch_t* out, int count, const int64_t* n, const int6
   for (size_t j = 0; j < b->large.size(); ++j) {
     const int i = b->large[j];
     cs_plan_t p = nullptr;
-    const cs_status st = cs_plan(&p, n[i], m[i], rows + b->moff[i], c + b->noff[i], s);
+    const cs_status st = (cs_status)plan_for_group(&p, n[i], m[i], rows + b->moff[i], c + b->noff[i], s);
     if (st != CS_OK) return fail(st);
     b->plans.push_back(p);
   }
   if (!b->large.empty()) {
     auto& G = b->grp;
     G.count = (int)b->large.size();
+    CS_B_TRY(init_col_multi_kernels());
+    CS_B_TRY(init_mid_multi_kernels());
     CS_B_TRY(cudaStreamCreateWithFlags(&G.cap, cudaStreamNonBlocking));
     CS_B_TRY(balloc(&G.desc, G.count));
     CS_B_TRY(balloc(&G.kps_i, G.count));

@@ -131,10 +131,11 @@ struct DynLayout {
   }
 };
 
-template <int LGL, int LGNV, bool VEC_FAST>
+// LGR: log2 of the leading radix (4: 16 values per thread, 3: 8).
+template <int LGL, int LGNV, bool VEC_FAST, int LGR = 4>
 struct StaticLayout {
   static constexpr bool kStatic = true;
-  static constexpr int kLgL = LGL, kLgNv = LGNV;
+  static constexpr int kLgL = LGL, kLgNv = LGNV, kLgR = LGR;
   __device__ __forceinline__ constexpr int LG() const { return LGL; }
   __device__ __forceinline__ constexpr int NV() const { return LGNV; }
   __device__ __forceinline__ constexpr bool VF() const { return VEC_FAST; }
@@ -144,7 +145,9 @@ struct StaticLayout {
   // Padded index split: pad(at(vec, idx)) = padV(vec) + padP(idx), and
   // padP(a + b) = padP(a) + padP(b) whenever b (or a) times the element
   // stride is a multiple of 16 -- so a stage's 16 reads / writes are one base
-  // plus compile-time offsets.  (Cols: vec < 2^LGNV <= 16 never carries.)
+  // plus compile-time offsets.  (Cols: vec < 2^LGNV <= 16 never carries.)  It
+  // also holds for a < 8 mod 16 and b a multiple of 8 (nothing carries past
+  // 16), which covers the radix-8 stages with Ls or L/R = 8.
   __device__ __forceinline__ static constexpr int padP(int idx) {
     return VEC_FAST ? ((idx << LGNV) + ((idx << LGNV) >> 4)) : (idx + (idx >> 4));
   }
@@ -159,7 +162,7 @@ struct StaticLayout {
 // j + r * (L / R): butterfly j, slot r.
 struct NoHook {
   static constexpr bool kPre = false, kPost = false;
-  __device__ __forceinline__ void begin(int, int) {}
+  __device__ __forceinline__ void begin(int, int, int) {}   // vec, j, the thread's butterfly number
   __device__ __forceinline__ float2 pre(int, int, int, int, float2 v) const { return v; }
   __device__ __forceinline__ float2 post(int, int, int, int, float2 v) { return v; }
 };
@@ -289,7 +292,7 @@ __device__ __forceinline__ void stockham_stage(float2* s, const LAY& lay, int lg
       const int j = js[i];
       const int k = j & (Ls - 1);
       if (H::kPre && first) {
-        hook.begin(vecs[i], j);
+        hook.begin(vecs[i], j, i);
 #pragma unroll
         for (int r = 0; r < R; ++r) v[i][r] = hook.pre(vecs[i], j, r, lgLR, v[i][r]);
       }
@@ -308,7 +311,7 @@ __device__ __forceinline__ void stockham_stage(float2* s, const LAY& lay, int lg
       }
       dft<R, DIR>(v[i]);
       const int base = ((j - k) << lgR) + k;   // in the last stage base == j, Ls == L/R
-      if (H::kPost && last && !(H::kPre && first)) hook.begin(vecs[i], j);
+      if (H::kPost && last && !(H::kPre && first)) hook.begin(vecs[i], j, i);
       // static layouts: Ls * stride is a multiple of 16 past the first stage,
       // and in the first stage base = 16 j is (radix 16), so the split holds
       float2* sb = s;
@@ -336,27 +339,49 @@ __device__ __forceinline__ void tile_fft(float2* s, const LAY& lay, const float2
                                          H& hook, const IN& in = IN{}, const OUT& out = OUT{}) {
   if constexpr (LAY::kStatic) {
     constexpr int LGL = LAY::kLgL;
-    constexpr int N16 = LGL / 4;      // radix-16 stages
-    constexpr int rem = LGL % 4;      // radix of the closing stage: 2^rem (none when 0)
-    constexpr int NST = N16 + (rem ? 1 : 0);
-    static_assert(NST >= 2, "a global source and sink need distinct first and last stages");
-    // with TWS, stage st (span 16^st) reads block st-1 of the stage-major table
-    int off = 0;
+    if constexpr (LAY::kLgR == 3) {
+      // radix 8 throughout, one closing radix-2 / 4 stage
+      constexpr int N8 = LGL / 3, rem8 = LGL % 3;
+      constexpr int NS8 = N8 + (rem8 ? 1 : 0);
+      static_assert(NS8 >= 2, "a global source and sink need distinct first and last stages");
+      int off8 = 0;
 #pragma unroll
-    for (int st = 0; st < N16; ++st) {
-      const float2* tws = TWS ? tw + off : tw;
-      if (st == 0)
-        stockham_stage<16, DIR, TILE, NT, TWS>(s, lay, 0, tws, lgLt, hook, in, SmemIO{});
-      else if (st == NST - 1)
-        stockham_stage<16, DIR, TILE, NT, TWS>(s, lay, 4 * st, tws, lgLt, hook, SmemIO{}, out);
-      else
-        stockham_stage<16, DIR, TILE, NT, TWS>(s, lay, 4 * st, tws, lgLt, hook);
-      if (st > 0) off += tw_rows(4) << (4 * st);
+      for (int st = 0; st < N8; ++st) {
+        const float2* tws = TWS ? tw + off8 : tw;
+        if (st == 0)
+          stockham_stage<8, DIR, TILE, NT, TWS>(s, lay, 0, tws, lgLt, hook, in, SmemIO{});
+        else if (st == NS8 - 1)
+          stockham_stage<8, DIR, TILE, NT, TWS>(s, lay, 3 * st, tws, lgLt, hook, SmemIO{}, out);
+        else
+          stockham_stage<8, DIR, TILE, NT, TWS>(s, lay, 3 * st, tws, lgLt, hook);
+        if (st > 0) off8 += tw_rows(3) << (3 * st);
+      }
+      const float2* tw8 = TWS ? tw + off8 : tw;
+      if constexpr (rem8 == 2) stockham_stage<4, DIR, TILE, NT, TWS>(s, lay, LGL - 2, tw8, lgLt, hook, SmemIO{}, out);
+      if constexpr (rem8 == 1) stockham_stage<2, DIR, TILE, NT, TWS>(s, lay, LGL - 1, tw8, lgLt, hook, SmemIO{}, out);
+    } else {
+      constexpr int N16 = LGL / 4;      // radix-16 stages
+      constexpr int rem = LGL % 4;      // radix of the closing stage: 2^rem (none when 0)
+      constexpr int NST = N16 + (rem ? 1 : 0);
+      static_assert(NST >= 2, "a global source and sink need distinct first and last stages");
+      // with TWS, stage st (span 16^st) reads block st-1 of the stage-major table
+      int off = 0;
+#pragma unroll
+      for (int st = 0; st < N16; ++st) {
+        const float2* tws = TWS ? tw + off : tw;
+        if (st == 0)
+          stockham_stage<16, DIR, TILE, NT, TWS>(s, lay, 0, tws, lgLt, hook, in, SmemIO{});
+        else if (st == NST - 1)
+          stockham_stage<16, DIR, TILE, NT, TWS>(s, lay, 4 * st, tws, lgLt, hook, SmemIO{}, out);
+        else
+          stockham_stage<16, DIR, TILE, NT, TWS>(s, lay, 4 * st, tws, lgLt, hook);
+        if (st > 0) off += tw_rows(4) << (4 * st);
+      }
+      const float2* twr = TWS ? tw + off : tw;
+      if constexpr (rem == 3) stockham_stage<8, DIR, TILE, NT, TWS>(s, lay, LGL - 3, twr, lgLt, hook, SmemIO{}, out);
+      if constexpr (rem == 2) stockham_stage<4, DIR, TILE, NT, TWS>(s, lay, LGL - 2, twr, lgLt, hook, SmemIO{}, out);
+      if constexpr (rem == 1) stockham_stage<2, DIR, TILE, NT, TWS>(s, lay, LGL - 1, twr, lgLt, hook, SmemIO{}, out);
     }
-    const float2* twr = TWS ? tw + off : tw;
-    if constexpr (rem == 3) stockham_stage<8, DIR, TILE, NT, TWS>(s, lay, LGL - 3, twr, lgLt, hook, SmemIO{}, out);
-    if constexpr (rem == 2) stockham_stage<4, DIR, TILE, NT, TWS>(s, lay, LGL - 2, twr, lgLt, hook, SmemIO{}, out);
-    if constexpr (rem == 1) stockham_stage<2, DIR, TILE, NT, TWS>(s, lay, LGL - 1, twr, lgLt, hook, SmemIO{}, out);
   } else {
     static_assert(!IN::kGlobal && !OUT::kGlobal, "run-time layouts use the shared tile only");
     int lgLs = 0;
@@ -377,11 +402,12 @@ __device__ __forceinline__ void tile_fft(float2* s, const LAY& lay, const float2
 }
 
 // Entries of the stage-major twiddle table of a length-L FFT: stage s >= 1
-// (span Ls, radix R) contributes tw_rows(log2 R) * Ls entries.
-__host__ __device__ constexpr int stage_tw_count(int lgL) {
+// (span Ls, radix R) contributes tw_rows(log2 R) * Ls entries.  lgRmax: log2
+// of the leading radix.
+__host__ __device__ constexpr int stage_tw_count(int lgL, int lgRmax = 4) {
   int n = 0, lgLs = 0;
   while (lgLs < lgL) {
-    const int lgR = (lgL - lgLs) >= 4 ? 4 : (lgL - lgLs);
+    const int lgR = (lgL - lgLs) >= lgRmax ? lgRmax : (lgL - lgLs);
     if (lgLs > 0) n += tw_rows(lgR) << lgLs;
     lgLs += lgR;
   }

@@ -19,8 +19,9 @@ struct Geo {
   int N, lgN, N1, lgN1, N2, lgN2;
   int G, lgG, col_ctas;
   int U, lgU, mid_ctas;
-  int tile;            // mid pass: complex values per CTA (4096 or 8192); threads = tile / 16
-  int col_tile;        // column pass: complex values per CTA (4096, or 8192 for N2 = 4096)
+  int tile;            // mid pass: complex values per CTA; threads = tile / 16 (tile / 8 with mid_r8)
+  int col_tile;        // column pass: complex values per CTA; threads = col_tile / 16 (/ 8 with col_r8)
+  int col_r8, mid_r8;  // 1: the pass runs 8 values per thread and radix-8 stages (small tiles, see make_geo)
   int twod;            // 1: 2D DFT of the N2 x N1 array (no four-step twiddle; pairs (k2, k1) ~ (-k2, -k1))
   const float2* tw1;   // exp(-2 pi i q / (2 N1)), q < 2 N1
   const float2* tw2;   // exp(-2 pi i q / N2),     q < N2
@@ -130,9 +131,9 @@ enum MidKind : int {
 cudaError_t launch_col(ColKind kind, const KParams& kp, cudaStream_t s);
 cudaError_t launch_mid(MidKind kind, const KParams& kp, cudaStream_t s);
 size_t pass_smem_bytes(int tile);
-cudaError_t init_pass_kernels();
-cudaError_t init_col_kernels();
-cudaError_t init_mid_kernels();
+// Shared-memory attributes of the pass kernels that geometry g launches.
+cudaError_t init_col_kernels(const Geo& g);
+cudaError_t init_mid_kernels(const Geo& g);
 // Grouped launches over many plans (batched solves, run-time shapes,
 // 4096-value tiles): CTA b runs tile map[b].y of the plan whose parameters
 // are kps[map[b].x] (both device arrays).
@@ -162,7 +163,7 @@ cudaError_t launch_fft64_2d(const double* c2, double2* a, double2* b, int64_t n0
                             cudaStream_t s);
 // Pair slots of the mid pass (spectrum tables' length).
 inline int64_t tab_count(const Geo& g) { return ((int64_t)(g.N2 >> 1) << g.lgN1) + (g.twod ? 2 : 1); }
-cudaError_t launch_stage_tw(float2* dst, int lgL, int count, cudaStream_t s);
+cudaError_t launch_stage_tw(float2* dst, int lgL, int lgRmax, cudaStream_t s);
 cudaError_t launch_tab_admm(const double2* chat, const Geo& g, int64_t n, float2* tabc,
                             double* abs2, cudaStream_t s);
 cudaError_t launch_tab_admm_b(const double* abs2, int count, int64_t n, double rho,
@@ -212,6 +213,9 @@ struct PlanView {
   GroupDesc desc;
 };
 PlanView plan_view(cs_plan_s* p);
+// A 1D plan whose passes use 4096-value tiles at every size (cs_plan's own
+// argument checks apply): the geometry of the grouped launches.
+int plan_for_group(cs_plan_s** out, int64_t n, int64_t m, const int64_t* rows, const double* c, void* stream);
 // Re-tabulate the plan's ADMM inverse spectrum for (rho, sigma) when it holds
 // another pair.
 cudaError_t plan_admm_table(cs_plan_s* p, double rho, double sigma, cudaStream_t s);

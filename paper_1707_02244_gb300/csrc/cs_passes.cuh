@@ -151,6 +151,18 @@ __device__ __forceinline__ void st2(float* p, int i, float2 v) {
 // block of every one of them.
 template <int KIND> struct Epi;
 
+// An epilogue with `Pre` splits in two: load() reads what it needs from
+// global memory (the solver state, the kept rows' y), apply() computes.  The
+// 8-value-per-thread tiles call load() for all their elements before the
+// inverse FFT starts, so that those reads are not waited for one stage after
+// the other; the 16-value tiles call it at the element (no registers to hold
+// the values).
+struct PreNone {};
+template <class E, class = void> struct HasPre : std::false_type {};
+template <class E> struct HasPre<E, std::void_t<typename E::Pre>> : std::true_type {};
+template <class E, class = void> struct PreOf { using T = PreNone; };
+template <class E> struct PreOf<E, std::void_t<typename E::Pre>> { using T = typename E::Pre; };
+
 template <> struct Epi<COL_LOAD> {
   static constexpr bool kRead = false, kFwd = true;
   __device__ static float2 apply(const KParams& kp, const CallArgs& a, float2, int p, int t, Acc&) {
@@ -188,14 +200,23 @@ template <> struct Epi<COL_MASK> {
 
 // r~ = M (P^T y - C x): residual of Algorithm 1 on the kept rows, zero off
 // them, so that the next product gives A^T r = C^T P^T r.
-template <> struct Epi<COL_RESIDUAL> {
-  static constexpr bool kRead = true, kFwd = true;
-  __device__ static float2 apply(const KParams& kp, const CallArgs&, float2 v, int p, int t, Acc& acc) {
+struct EpiRows2 {   // the kept rows among elements 2t, 2t + 1 and their y
+  struct Pre { uint32_t mm; float y0, y1; };
+  __device__ static Pre load(const KParams& kp, const CallArgs&, int p, int t, const Acc& acc) {
     RowSel rs{acc.smask, acc.spref, acc.wbase};
     int i0;
-    const uint32_t mm = rs.get2(t, i0);
-    const float r0 = (mm & 1u) ? __ldg(kp.pp.ys + i0) - v.x : 0.f;
-    const float r1 = (mm & 2u) ? __ldg(kp.pp.ys + i0 + (int)(mm & 1u)) - v.y : 0.f;
+    Pre q;
+    q.mm = rs.get2(t, i0);
+    q.y0 = (q.mm & 1u) ? __ldg(kp.pp.ys + i0) : 0.f;
+    q.y1 = (q.mm & 2u) ? __ldg(kp.pp.ys + i0 + (int)(q.mm & 1u)) : 0.f;
+    return q;
+  }
+};
+template <> struct Epi<COL_RESIDUAL> : EpiRows2 {
+  static constexpr bool kRead = true, kFwd = true;
+  __device__ static float2 apply(const KParams& kp, const CallArgs&, float2 v, int p, int t, Acc& acc, const Pre& q) {
+    const float r0 = (q.mm & 1u) ? q.y0 - v.x : 0.f;
+    const float r1 = (q.mm & 2u) ? q.y1 - v.y : 0.f;
     acc.v[ST_R2] = fmaf(r0, r0, fmaf(r1, r1, acc.v[ST_R2]));
     return make_float2(r0, r1);
   }
@@ -208,9 +229,13 @@ template <> struct Epi<COL_RESIDUAL> {
 // stores to x (that might otherwise alias them).
 template <bool FWD> struct EpiIsta {
   static constexpr bool kRead = true, kFwd = FWD;
-  __device__ static float2 apply(const KParams& kp, const CallArgs& a, float2 g, int p, int t, Acc& acc) {
+  using Pre = float2;
+  __device__ static Pre load(const KParams&, const CallArgs& a, int p, int t, const Acc&) {
+    return __ldg(reinterpret_cast<const float2*>(a.x) + t);
+  }
+  __device__ static float2 apply(const KParams& kp, const CallArgs& a, float2 g, int p, int t, Acc& acc,
+                                 const Pre& xo) {
     float2* x = reinterpret_cast<float2*>(a.x);
-    const float2 xo = __ldg(x + t);
     float2 xn;
     xn.x = soft(fmaf(a.tau, g.x, xo.x), a.thr);
     xn.y = soft(fmaf(a.tau, g.y, xo.y), a.thr);
@@ -257,14 +282,23 @@ template <> struct Epi<COL_ADMM_INIT> {
 // v <- v + mu; the next x-update reads (v) + i (z - nu).
 template <bool FWD, bool SEG = false> struct EpiAdmm {
   static constexpr bool kRead = true, kFwd = FWD;
-  __device__ static float2 apply(const KParams& kp, const CallArgs& a, float2 xc, int p, int t, Acc& acc) {
+  struct Pre { bool on; float yv, mu, nu; };
+  __device__ static Pre load(const KParams& kp, const CallArgs& a, int p, int t, const Acc& acc) {
     RowSel rs{acc.smask, acc.spref, acc.wbase};
     int iy;
-    const bool on = rs.get(t, iy);
-    const float yv = on ? __ldg(kp.pp.ys + iy) : 0.f;
-    const float x = xc.x, cx = xc.y;
+    Pre q;
+    q.on = rs.get(t, iy);
+    q.yv = q.on ? __ldg(kp.pp.ys + iy) : 0.f;
     // read-once / write-once per element by its own thread: read-only path (as EpiIsta)
-    const float mu = __ldg(a.mu + t), nu = __ldg(a.nu + t);
+    q.mu = __ldg(a.mu + t);
+    q.nu = __ldg(a.nu + t);
+    return q;
+  }
+  __device__ static float2 apply(const KParams& kp, const CallArgs& a, float2 xc, int p, int t, Acc& acc,
+                                 const Pre& q) {
+    const bool on = q.on;
+    const float yv = q.yv, mu = q.mu, nu = q.nu;
+    const float x = xc.x, cx = xc.y;
     const float d = on ? a.d_on : a.d_off;
     const float v = d * fmaf(a.rho, cx - mu, yv);
     const float z = soft(x + nu, a.thr);
@@ -372,14 +406,12 @@ template <> struct Epi<COL_LOADT> {
   }
 };
 
-template <> struct Epi<COL_RES_SAVE> {
+template <> struct Epi<COL_RES_SAVE> : EpiRows2 {
   static constexpr bool kRead = true, kFwd = true;
-  __device__ static float2 apply(const KParams& kp, const CallArgs& a, float2 v, int p, int t, Acc& acc) {
-    RowSel rs{acc.smask, acc.spref, acc.wbase};
-    int i0;
-    const uint32_t mm = rs.get2(t, i0);
-    const float r0 = (mm & 1u) ? __ldg(kp.pp.ys + i0) - v.x : 0.f;
-    const float r1 = (mm & 2u) ? __ldg(kp.pp.ys + i0 + (int)(mm & 1u)) - v.y : 0.f;
+  __device__ static float2 apply(const KParams& kp, const CallArgs& a, float2 v, int p, int t, Acc& acc,
+                                 const Pre& q) {
+    const float r0 = (q.mm & 1u) ? q.y0 - v.x : 0.f;
+    const float r1 = (q.mm & 2u) ? q.y1 - v.y : 0.f;
     const float2 r = make_float2(r0, r1);
     st2(a.v, t, r);
     return r;
@@ -388,8 +420,9 @@ template <> struct Epi<COL_RES_SAVE> {
 
 template <> struct Epi<COL_ISTA_SEG> {
   static constexpr bool kRead = true, kFwd = true;
-  __device__ static float2 apply(const KParams&, const CallArgs& a, float2 g, int p, int t, Acc&) {
-    const float2 xo = ld2(a.x, t);
+  using Pre = float2;
+  __device__ static Pre load(const KParams&, const CallArgs& a, int p, int t, const Acc&) { return ld2(a.x, t); }
+  __device__ static float2 apply(const KParams&, const CallArgs& a, float2 g, int p, int t, Acc&, const Pre& xo) {
     const float2 xn = make_float2(soft(fmaf(a.tau, g.x, xo.x), a.thr), soft(fmaf(a.tau, g.y, xo.y), a.thr));
     st2(a.z, t, xn);
     return xn;
@@ -444,9 +477,13 @@ template <> struct Epi<COL_LOAD2> {
   }
 };
 
-template <int TILE> struct Cfg {
-  static constexpr int NT = TILE / EPT;                 // threads per CTA
-  static constexpr int MINB = 65536 / (64 * NT);        // mid pass: CTAs per SM at <= 64 registers
+// VPT: complex values per thread (16, or 8 for the radix-8 tiles).
+constexpr int VPT8 = 8;
+template <int TILE, int VPT = EPT> struct Cfg {
+  static constexpr int NT = TILE / VPT;                 // threads per CTA
+  // CTAs per SM: 1024 threads at <= 64 registers; the radix-8 tiles never
+  // fill the chip, so they take up to ~100 registers for their early loads
+  static constexpr int MINB = VPT == VPT8 ? (640 / NT < 1 ? 1 : 640 / NT) : 65536 / (64 * NT);
   static constexpr int NLD = TILE / (2 * NT);           // float4 loads per thread per tile
 };
 
@@ -460,10 +497,10 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename K>
-cudaError_t launch_k(K kern, int grid, int tile, const KParams& kp, cudaStream_t s, int smem_mult = 1) {
+cudaError_t launch_k(K kern, int grid, int tile, int vpt, const KParams& kp, cudaStream_t s, int smem_mult = 1) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(tile / EPT);
+  cfg.blockDim = dim3(tile / vpt);
   cfg.dynamicSmemBytes = smem_mult * pass_smem_bytes(tile);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -487,6 +524,7 @@ cudaError_t set_smem(K kern, int tile, int ctas, int smem_mult = 1) {
   if (e != cudaSuccess) return e;
   const size_t per_cta = dyn + fa.sharedSizeBytes + 1024;
   int pct = (int)((per_cta * ctas * 100 + 228 * 1024 - 1) / (228 * 1024));
+  if (ctas < 1) pct = 50;   // radix-8 tiles: one carveout for all of them, so no SM reconfigures between passes
   if (pct > 100) pct = 100;
   return cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
 }
