@@ -61,6 +61,17 @@ struct cs_plan_s {
   std::map<uint64_t, int> graph_nodes;
   std::map<uint64_t, cudaGraphExec_t> graphs;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+  // Single-CTA solves (n <= 8192; ADMM n <= 4096): tables in natural order
+  bool small_i = false, small_a = false;
+  int lgn = 0;
+  struct Small {
+    float4* tA = nullptr;
+    float2 *tB = nullptr, *tc = nullptr, *tw_i = nullptr, *tw_a = nullptr;
+    double* abs2 = nullptr;
+    float* tb = nullptr;
+  } sml;
+  CallArgs last_ca{};              // arguments of the last single-CTA solve: cs_profile_pass sends them first
+  bool ca_stale = false;
   // unrolled-ISTA gradient (cs_grad): allocated at the first call, grown on demand
   struct Grad {
     int ck_cap = 0, seg_cap = 0;
@@ -220,6 +231,9 @@ void free_plan(cs_plan_s* p) {
                   p->dense, p->dense2, p->dense3};
   for (void* b : bufs)
     if (b) cudaFree(b);
+  void* sbufs[] = {p->sml.tA, p->sml.tB, p->sml.tc, p->sml.tw_i, p->sml.tw_a, p->sml.abs2, p->sml.tb};
+  for (void* b : sbufs)
+    if (b) cudaFree(b);
   void* gbufs[] = {p->gr.ckpt, p->gr.seg, p->gr.rseg, p->gr.g, p->gr.w, p->gr.q, p->gr.dy, p->gr.W2, p->gr.gacc,
                    p->gr.gpart, p->gr.ca};
   for (void* b : gbufs)
@@ -361,19 +375,21 @@ cudaError_t run_chunk(cs_plan_s* p, SolveKind kind, int len, bool final_chunk, b
 
 // Iterate in chunks of check_every; with a monitor tolerance, stop at the
 // first check point whose NMSE meets it.
-cudaError_t solve_loop(cs_plan_s* p, SolveKind kind, int iters, int* iters_run, int* converged,
-                       bool need_stats) {
+// step(done, len, final chunk, statistics) enqueues iterations done .. done +
+// len - 1; at most `most` in one chunk when nobody watches.
+template <class F>
+cudaError_t solve_loop(cs_plan_s* p, int iters, int* iters_run, int* converged, bool need_stats, int most, F&& step) {
   *iters_run = 0;
   *converged = 0;
-  const int ce = p->check_every;
   const bool watch = p->xtrue != nullptr && p->tol > 0.0;
+  const int ce = watch || most < p->check_every ? p->check_every : most;
   int done = 0;
   while (done < iters) {
     const int len = (iters - done) < ce ? (iters - done) : ce;
     const bool final_chunk = done + len == iters;
     // the statistics of a check point are formed where somebody reads them:
     // by the monitor at every one, else by the caller's record at the last
-    cudaError_t e = run_chunk(p, kind, len, final_chunk, watch || (final_chunk && need_stats));
+    cudaError_t e = step(done, len, final_chunk, watch || (final_chunk && need_stats));
     if (e != cudaSuccess) return e;
     done += len;
     if (watch && !final_chunk) {
@@ -413,6 +429,44 @@ void fill_stats(const cs_plan_s* p, cs_stats* st, int iters_run, int converged, 
   st->objective = 0.5 * h[ST_R2] + lambda * h[ST_L1];
   st->launches = p->launches;
   (void)admm;
+}
+
+// Longest single-CTA launch (iterations): tens of milliseconds.
+constexpr int SMALL_CHUNK = 10000;
+
+SmallArgs small_args(const cs_plan_s* p, bool admm) {
+  SmallArgs a{};
+  const Geo& g = admm ? p->ga : p->gi;
+  a.tA = p->sml.tA;
+  a.tB = p->sml.tB;
+  a.tc = p->sml.tc;
+  a.tb = p->sml.tb;
+  a.tw = admm ? p->sml.tw_a : p->sml.tw_i;
+  a.rows = p->rows32;
+  a.m = (int)p->m;
+  a.status = p->status;
+  a.xtrue = p->xtrue ? (admm ? p->xt_a : p->xt_i) : nullptr;
+  a.lgN1 = g.lgN1;
+  a.lgN2 = g.lgN2;
+  a.lgG = g.lgG;
+  return a;
+}
+
+// B's spectrum 1 / (n (rho |c^|^2 + sigma)) of the plan, tabulated when it
+// holds another pair.
+cudaError_t admm_table(cs_plan_s* p, double rho, double sigma, cudaStream_t s, int* launches) {
+  if (rho == p->b_rho && sigma == p->b_sigma) return cudaSuccess;
+  cudaError_t e = launch_tab_admm_b(p->abs2, (int)tab_count(p->ga), p->n, rho, sigma, p->tab_admm_b, s);
+  if (launches) *launches += 1;
+  if (e == cudaSuccess && p->small_a) {
+    e = launch_tab_admm_b(p->sml.abs2, (int)(p->n / 2 + 1), p->n, rho, sigma, p->sml.tb, s);
+    if (launches) *launches += 1;
+  }
+  if (e == cudaSuccess) {
+    p->b_rho = rho;
+    p->b_sigma = sigma;
+  }
+  return e;
 }
 
 bool valid_ptr(const void* q) { return q != nullptr && ((uintptr_t)q & 7u) == 0; }
@@ -568,9 +622,23 @@ cs_status build_plan(cs_plan_t* out, int64_t n0, int64_t n1, int64_t m, const in
     CS_PLAN_TRY(launch_tab_ista(chat, p->gi, n, p->tab_ista, s));
     CS_PLAN_TRY(launch_tab_admm(chat, p->ga, n, p->tab_admm_c, p->abs2, s));
   }
-  CS_PLAN_TRY(launch_tab_admm_b(p->abs2, (int)tab_count(p->ga), n, 1.0, 1.0, p->tab_admm_b, s));
-  p->b_rho = 1.0;
-  p->b_sigma = 1.0;
+  p->lgn = lgn;
+  p->small_i = !twod && small_tiles && lgn - 1 <= SMALL_LG_MAX;
+  p->small_a = !twod && small_tiles && lgn <= SMALL_LG_MAX;
+  if (p->small_i) {
+    CS_PLAN_TRY(dalloc(&p->sml.tA, n / 4 + 1));
+    CS_PLAN_TRY(dalloc(&p->sml.tB, n / 4 + 1));
+    CS_PLAN_TRY(dalloc(&p->sml.tw_i, small_tw_count(lgn - 1)));
+    if (p->small_a) {
+      CS_PLAN_TRY(dalloc(&p->sml.tc, n / 2 + 1));
+      CS_PLAN_TRY(dalloc(&p->sml.abs2, n / 2 + 1));
+      CS_PLAN_TRY(dalloc(&p->sml.tb, n / 2 + 1));
+      CS_PLAN_TRY(dalloc(&p->sml.tw_a, small_tw_count(lgn)));
+    }
+    CS_PLAN_TRY(launch_small_tables(chat, n, lgn, p->sml.tA, p->sml.tB, p->sml.tc, p->sml.abs2, p->sml.tw_i,
+                                    p->sml.tw_a, s));
+  }
+  CS_PLAN_TRY(admm_table(p, 1.0, 1.0, s, nullptr));
   CS_PLAN_TRY(launch_build_mask(d_rows, m, n, p->gi, 1, p->si.mask, p->status, s));
   CS_PLAN_TRY(launch_build_mask(d_rows, m, n, p->ga, 0, p->sa.mask, p->status, s));
   CS_PLAN_TRY(launch_prefix(p->si.mask, words, p->si.prefix, s));
@@ -615,11 +683,18 @@ cs_status cs_status_sync(cs_plan_t p) {
 
 cs_status cs_forward(cs_plan_t p, const float* x, float* y) {
   if (!p || !valid_ptr(x) || !y) return CS_ERR_ARG;
+  cudaStream_t s = p->stream;
+  p->ista_args = p->admm_args = false;
+  if (p->small_i) {
+    SmallArgs sa = small_args(p, false);
+    sa.x = const_cast<float*>(x);
+    sa.yo = y;
+    CS_TRY(launch_small(SMALL_FWD, p->lgn - 1, sa, s));
+    return CS_OK;
+  }
   CallArgs a{};
   a.src = x;
   a.dst = p->dense;
-  cudaStream_t s = p->stream;
-  p->ista_args = p->admm_args = false;
   CS_TRY(launch_set_args(a, p->ca, s));
   CS_TRY(launch_col(COL_LOAD, kparams(p, p->gi, 0), s));
   CS_TRY(launch_mid(MID_FWD, kparams(p, p->gi, 0), s));
@@ -631,6 +706,14 @@ cs_status cs_forward(cs_plan_t p, const float* x, float* y) {
 cs_status cs_adjoint(cs_plan_t p, const float* r, float* x) {
   if (!p || !r || !valid_ptr(x)) return CS_ERR_ARG;
   cudaStream_t s = p->stream;
+  if (p->small_i) {
+    p->ista_args = p->admm_args = false;
+    SmallArgs sa = small_args(p, false);
+    sa.x = x;
+    sa.y = r;
+    CS_TRY(launch_small(SMALL_ADJ, p->lgn - 1, sa, s));
+    return CS_OK;
+  }
   CS_TRY(cudaMemsetAsync(p->dense, 0, p->n * sizeof(float), s));
   CS_TRY(launch_scatter_rows(r, p->rows32, p->m, p->dense, s));
   CallArgs a{};
@@ -648,6 +731,17 @@ cs_status cs_opnorm2(cs_plan_t p, int iters, double* L) {
   if (!p || !L || iters < 1) return CS_ERR_ARG;
   cudaStream_t s = p->stream;
   CS_TRY(launch_power_init(p->dense2, p->n, s));
+  if (p->small_i) {
+    p->ista_args = p->admm_args = false;
+    SmallArgs sa = small_args(p, false);
+    sa.x = p->dense2;
+    sa.stats = p->stats;
+    sa.iters = iters;
+    CS_TRY(launch_small(SMALL_POWER, p->lgn - 1, sa, s));
+    CS_TRY(read_back(p));
+    *L = p->host_stats[ST_DX2];
+    return latched_status(p);
+  }
   CS_TRY(launch_norm2(p->dense2, p->n, p->partials, p->stats + ST_X2, s));
   CallArgs a{};
   a.src = p->dense2;
@@ -702,17 +796,37 @@ cs_status cs_ista(cs_plan_t p, const float* y, float lambda, float tau, int iter
   a.thr = (float)((double)tau * (double)lambda);
   a.tau = tau;
   p->launches = 0;
-  CS_TRY(launch_set_args(a, p->ca, s));
-  CS_TRY(launch_scatter_y(y, p->si.pos, p->m, p->si.ys, p->status, s));
-  p->launches += 2;
   p->ista_args = true;
   p->admm_args = false;
   int run = 0, conv = 0;
-  if (iters > 0) {
+  if (p->small_i && iters > 0) {
+    SmallArgs sa = small_args(p, false);
+    sa.y = y;
+    sa.x = x;
+    sa.thr = a.thr;
+    sa.tau = tau;
+    p->last_ca = a;
+    p->ca_stale = true;
+    CS_TRY(solve_loop(p, iters, &run, &conv, stats != nullptr, SMALL_CHUNK,
+                      [&](int, int len, bool, bool st) {
+                        sa.iters = len;
+                        sa.stats = st ? p->stats : nullptr;
+                        p->launches += 1;
+                        return launch_small(SMALL_ISTA, p->lgn - 1, sa, s);
+                      }));
+  } else {
+    p->ca_stale = false;
+    CS_TRY(launch_set_args(a, p->ca, s));
+    CS_TRY(launch_scatter_y(y, p->si.pos, p->m, p->si.ys, p->status, s));
+    p->launches += 2;
+  }
+  if (!p->small_i && iters > 0) {
     CS_TRY(launch_to_tile(x, p->xi_t, p->gi, 1, s));
     CS_TRY(launch_col(COL_LOAD, kparams(p, p->gi, 0), s));
     p->launches += 2;
-    CS_TRY(solve_loop(p, K_ISTA, iters, &run, &conv, stats != nullptr));
+    CS_TRY(solve_loop(p, iters, &run, &conv, stats != nullptr, 0, [&](int, int len, bool fin, bool st) {
+      return run_chunk(p, K_ISTA, len, fin, st);
+    }));
     CS_TRY(launch_from_tile(p->xi_t, x, p->gi, 1, s));
     p->launches += 1;
   }
@@ -746,7 +860,8 @@ cs_status admm_impl(cs_plan_t p, const float* y, float lambda, const cs_admm_par
   p->launches = 0;
   float* tiled[4] = {p->av, p->az, p->amu, p->anu};
   float* natural[4] = {v, z, mu, nu};
-  for (int i = 0; i < 4; ++i) {
+  const bool small = p->small_a && iters > 0;
+  for (int i = 0; i < 4 && !small; ++i) {
     if (warm) {
       CS_TRY(launch_to_tile(natural[i], tiled[i], p->ga, 0, s));
       p->launches += 1;
@@ -754,12 +869,7 @@ cs_status admm_impl(cs_plan_t p, const float* y, float lambda, const cs_admm_par
       CS_TRY(cudaMemsetAsync(tiled[i], 0, nb, s));
     }
   }
-  if (prm->rho != p->b_rho || prm->sigma != p->b_sigma) {
-    CS_TRY(launch_tab_admm_b(p->abs2, (int)tab_count(p->ga), p->n, prm->rho, prm->sigma, p->tab_admm_b, s));
-    p->launches += 1;
-    p->b_rho = prm->rho;
-    p->b_sigma = prm->sigma;
-  }
+  CS_TRY(admm_table(p, prm->rho, prm->sigma, s, &p->launches));
   CallArgs a{};
   a.x = p->ax;
   a.z = p->az;
@@ -774,21 +884,54 @@ cs_status admm_impl(cs_plan_t p, const float* y, float lambda, const cs_admm_par
   a.tau2 = (float)prm->tau2;
   a.d_on = (float)(1.0 / (1.0 + prm->rho));
   a.d_off = (float)(1.0 / prm->rho);
-  CS_TRY(launch_set_args(a, p->ca, s));
-  CS_TRY(launch_scatter_y(y, p->sa.pos, p->m, p->sa.ys, p->status, s));
-  p->launches += 2;
   p->admm_args = true;
   p->ista_args = false;
   int run = 0, conv = 0;
-  if (iters > 0) {
+  if (small) {
+    p->last_ca = a;
+    p->ca_stale = true;
+    SmallArgs sa = small_args(p, true);
+    sa.y = y;
+    sa.thr = a.thr;
+    sa.rho = a.rho;
+    sa.sigma = a.sigma;
+    sa.tau1 = a.tau1;
+    sa.tau2 = a.tau2;
+    sa.d_on = a.d_on;
+    sa.d_off = a.d_off;
+    // a chunk that another one may follow leaves its state in the caller's
+    // vectors, or in the plan's where the caller takes none
+    const bool watch = p->xtrue != nullptr && p->tol > 0.0;
+    CS_TRY(solve_loop(p, iters, &run, &conv, stats != nullptr, SMALL_CHUNK, [&](int done, int len, bool fin, bool st) {
+      const bool carry = watch || !fin || done > 0;
+      sa.v = v ? v : carry ? p->av : nullptr;
+      sa.z = z ? z : carry ? p->az : nullptr;
+      sa.mu = mu ? mu : carry ? p->amu : nullptr;
+      sa.nu = nu ? nu : carry ? p->anu : nullptr;
+      sa.x = x;
+      sa.warm = warm || done > 0;
+      sa.iters = len;
+      sa.stats = st ? p->stats : nullptr;
+      p->launches += 1;
+      return launch_small(SMALL_ADMM, p->lgn, sa, s);
+    }));
+  } else {
+    p->ca_stale = false;
+    CS_TRY(launch_set_args(a, p->ca, s));
+    CS_TRY(launch_scatter_y(y, p->sa.pos, p->m, p->sa.ys, p->status, s));
+    p->launches += 2;
+  }
+  if (iters > 0 && !small) {
     CS_TRY(launch_col(COL_ADMM_INIT, kparams(p, p->ga, 0), s));
     p->launches += 1;
-    CS_TRY(solve_loop(p, K_ADMM, iters, &run, &conv, stats != nullptr));
+    CS_TRY(solve_loop(p, iters, &run, &conv, stats != nullptr, 0, [&](int, int len, bool fin, bool st) {
+      return run_chunk(p, K_ADMM, len, fin, st);
+    }));
   }
   float* outs_t[5] = {p->av, p->az, p->amu, p->anu, p->ax};
   float* outs_n[5] = {v, z, mu, nu, iters > 0 ? x : nullptr};
   for (int i = 0; i < 5; ++i) {
-    if (!outs_n[i]) continue;
+    if (small || !outs_n[i]) continue;
     CS_TRY(launch_from_tile(outs_t[i], outs_n[i], p->ga, 0, s));
     p->launches += 1;
   }
@@ -827,6 +970,10 @@ cs_status cs_profile_pass(cs_plan_t p, int pass_id, int reps) {
   if (pass_id <= 3 && !p->ista_args) return CS_ERR_ARG;
   if (pass_id >= 4 && !p->admm_args) return CS_ERR_ARG;
   cudaStream_t s = p->stream;
+  if (p->ca_stale) {
+    CS_TRY(launch_set_args(p->last_ca, p->ca, s));
+    p->ca_stale = false;
+  }
   for (int r = 0; r < reps; ++r) {
     switch (pass_id) {
       case 0: CS_TRY(launch_mid(MID_FWD, kparams(p, p->gi, 0), s)); break;
@@ -1133,12 +1280,7 @@ extern "C" cs_status cs_grad_admm(cs_plan_t p, const float* y, float lambda, con
   const int Kc = G.seg_cap;
   const size_t n = (size_t)p->n, nb = n * sizeof(float);
   p->launches = 0;
-  if (prm->rho != p->b_rho || prm->sigma != p->b_sigma) {
-    CS_TRY(launch_tab_admm_b(p->abs2, (int)tab_count(p->ga), p->n, prm->rho, prm->sigma, p->tab_admm_b, s));
-    p->launches += 1;
-    p->b_rho = prm->rho;
-    p->b_sigma = prm->sigma;
-  }
+  CS_TRY(admm_table(p, prm->rho, prm->sigma, s, &p->launches));
   CallArgs a{};
   a.x = p->ax;
   a.z = p->az;
@@ -1265,13 +1407,7 @@ PlanView plan_view(cs_plan_s* p) {
 }
 
 cudaError_t plan_admm_table(cs_plan_s* p, double rho, double sigma, cudaStream_t s) {
-  if (rho == p->b_rho && sigma == p->b_sigma) return cudaSuccess;
-  cudaError_t e = launch_tab_admm_b(p->abs2, (int)tab_count(p->ga), p->n, rho, sigma, p->tab_admm_b, s);
-  if (e == cudaSuccess) {
-    p->b_rho = rho;
-    p->b_sigma = sigma;
-  }
-  return e;
+  return admm_table(p, rho, sigma, s, nullptr);
 }
 
 }  // namespace csk

@@ -193,6 +193,35 @@ cudaError_t launch_power_init(float* u, int64_t n, cudaStream_t s);
 // out[0] = scale * sum(v[0 .. count)), summed in a fixed order in FP64.
 cudaError_t launch_sum_scaled(const double* v, int count, float scale, float* out, cudaStream_t s);
 
+// Single-CTA solves and products of short transforms (cs_small.cu): packed
+// length N = n/2 for ISTA, the power iteration and the products, N = n for
+// ADMM, N = 2^lgN <= 4096.  All vectors in natural order.
+constexpr int SMALL_LG_MAX = 12;
+enum SmallKind : int { SMALL_ISTA, SMALL_ADMM, SMALL_POWER, SMALL_FWD, SMALL_ADJ };
+struct SmallArgs {
+  const float4* tA;        // pair operator of the packed geometry, k in [0, N/2] (tA, tB)
+  const float2* tB;
+  const float2* tc;        // ADMM: c^_k and b^_k / n, k in [0, n/2]
+  const float* tb;
+  const float2* tw;        // stage twiddles
+  const int32_t* rows;     // rows of Omega in the caller's order
+  int m;
+  const float* y;          // y (solves), r (A^T r)
+  float* yo;               // A x
+  float *x, *z, *mu, *nu, *v;   // ISTA: x; ADMM: the state (null: not returned)
+  const float* xtrue;      // monitor ground truth in the plan's tile order, or null
+  int lgN1, lgN2, lgG;     // of the geometry xtrue is tiled for
+  double* stats;           // NSTAT sums of the last iteration, or null
+  int* status;
+  int iters, warm;
+  float thr, tau, rho, sigma, tau1, tau2, d_on, d_off;
+};
+cudaError_t launch_small(SmallKind kind, int lgN, const SmallArgs& a, cudaStream_t s);
+int small_tw_count(int lgN);
+// Tables of a plan of n = 2^lgn from its FP64 spectrum (tc, abs2, tw_a null: no ADMM).
+cudaError_t launch_small_tables(const double2* chat, int64_t n, int lgn, float4* tA, float2* tB, float2* tc,
+                                double* abs2, float2* tw_i, float2* tw_a, cudaStream_t s);
+
 // One plan of a grouped (batched) solve: what the grouped element-wise
 // kernels need of it.
 struct GroupDesc {

@@ -1,0 +1,201 @@
+// One CTA holds the whole FFT of a short transform: building blocks of the
+// solvers for n <= 8192 (cs_small.cu).
+//
+// N = 2^LG complex values, E per thread, kept in registers between the
+// stages.  A product with C is  forward FFT -> operator on the pairs
+// (k, N - k) -> inverse FFT, with radices R1 = E first and RL = E/2 last in
+// the forward direction and the same in reverse order on the way back:
+//   - the last inverse stage leaves elements tid + r N/R1 with thread tid,
+//     which are the inputs of its first forward stage, so the solver's
+//     element-wise step and the turn to the next product need no exchange;
+//   - thread tid runs butterflies j = tid and M - tid (M = N/RL; thread 0:
+//     0 and M/2) of the last forward stage.  Output r of butterfly j is
+//     frequency j + r M and its mirror is output RL-1-r of butterfly M - j
+//     (butterfly 0: RL - r of itself), so both members of every pair are
+//     in one thread and the operator and the first inverse stage (the same
+//     butterflies) work in registers.
+// A product then costs one exchange through shared memory per stage boundary
+// that is left: 2 (NS - 1) for NS stages, one barrier each (two buffers).
+#pragma once
+
+#include "cs_fft.cuh"
+
+namespace csk {
+
+// Shape of the transform.  8 values per thread up to N = 256, 16 above (more
+// threads against fewer exchanges).
+template <int LG> struct SmallShape {
+  static constexpr int kLgE = LG <= 8 ? 3 : 4;
+  static constexpr int E = 1 << kLgE;
+  static constexpr int N = 1 << LG;
+  static constexpr int NA = N / E;                     // threads that hold values
+  static constexpr int NT = NA < 32 ? 32 : NA;         // threads launched
+  static constexpr int kLg1 = kLgE, kLgL = kLgE - 1;   // first and last forward radix
+  static constexpr int kLgM = LG - kLg1 - kLgL;        // what is left for the middle stages
+  static constexpr int kLgM1 = kLgM > kLgE ? (kLgM + 1) / 2 : kLgM;
+  static constexpr int kLgM2 = kLgM - kLgM1;
+  static_assert(kLgM >= 0 && kLgM1 <= kLgE && kLgM2 <= kLgE, "radices");
+  // twiddle blocks: forward middle 1, middle 2, last; inverse middle 2, middle 1, last (radix R1)
+  static constexpr int kF1 = 0;
+  static constexpr int kF2 = kF1 + (kLgM1 ? tw_rows(kLgM1) << kLg1 : 0);
+  static constexpr int kFL = kF2 + (kLgM2 ? tw_rows(kLgM2) << (kLg1 + kLgM1) : 0);
+  static constexpr int kI2 = kFL + (tw_rows(kLgL) << (LG - kLgL));
+  static constexpr int kI1 = kI2 + (kLgM2 ? tw_rows(kLgM2) << kLgL : 0);
+  static constexpr int kIL = kI1 + (kLgM1 ? tw_rows(kLgM1) << (kLgL + kLgM2) : 0);
+  static constexpr int kTw = kIL + (tw_rows(kLg1) << (LG - kLg1));
+};
+
+// The same description for the host and the table kernel: stage b holds
+// rows r(row) of w_{Ls R}^(r k) at off + row Ls + k.
+struct SmallTwStages {
+  int count;
+  int off[6], lgLs[6], lgR[6];
+  int total;
+};
+template <int LG> SmallTwStages small_tw_stages() {
+  using S = SmallShape<LG>;
+  SmallTwStages d{};
+  auto add = [&](int off, int lgLs, int lgR) {
+    if (lgR == 0) return;
+    d.off[d.count] = off;
+    d.lgLs[d.count] = lgLs;
+    d.lgR[d.count++] = lgR;
+  };
+  add(S::kF1, S::kLg1, S::kLgM1);
+  add(S::kF2, S::kLg1 + S::kLgM1, S::kLgM2);
+  add(S::kFL, LG - S::kLgL, S::kLgL);
+  add(S::kI2, S::kLgL, S::kLgM2);
+  add(S::kI1, S::kLgL + S::kLgM2, S::kLgM1);
+  add(S::kIL, LG - S::kLg1, S::kLg1);
+  d.total = S::kTw;
+  return d;
+}
+
+// padP(a + b) = padP(a) + padP(b) for every base and offset of a stage: the
+// strides are powers of two, so the parts below 16 never carry.
+__host__ __device__ constexpr int padP(int i) { return i + (i >> 4); }
+
+template <int LG> __host__ __device__ constexpr int small_buf() { return padP(1 << LG); }   // float2 per exchange buffer
+
+// One middle stage (span 2^LGLS, radix 2^LGR) from buffer a to buffer b.
+template <int LG, int LGLS, int LGR, int DIR>
+__device__ __forceinline__ void small_mid(const float2* a, float2* b, const float2* tw) {
+  using S = SmallShape<LG>;
+  constexpr int R = 1 << LGR, LS = 1 << LGLS, B = S::E / R, ST = S::N / R;
+  if (threadIdx.x < S::NA) {
+    float2 v[B][R];
+#pragma unroll
+    for (int i = 0; i < B; ++i) {
+      const float2* q = a + padP(threadIdx.x + i * S::NA);
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[i][r] = q[padP(r * ST)];
+    }
+#pragma unroll
+    for (int i = 0; i < B; ++i) {
+      const int j = threadIdx.x + i * S::NA, k = j & (LS - 1);
+      stage_twiddle<R, DIR>(v[i], tw, LS, k);
+      dft<R, DIR>(v[i]);
+      float2* q = b + padP(((j - k) << LGR) + k);
+#pragma unroll
+      for (int r = 0; r < R; ++r) q[padP(r * LS)] = v[i][out_slot<R>(r)];
+    }
+  }
+  __syncthreads();
+}
+
+// v (element tid + r N/R1 in v[r]) -> inverse FFT of op(forward FFT of v),
+// unnormalised, in the same order.  op(k, za, zb) is applied to every pair
+// (k, N - k), k <= N/2; for the self-pairs k = 0 and N/2 za and zb hold the
+// same value and za is kept.  S0, S1: exchange buffers; on return S0 and S1
+// may still be read by other threads of the CTA only in the way the next call
+// allows (it writes S0 first, whose last reader is behind a barrier).
+template <int LG, class OP>
+__device__ __forceinline__ void small_conv(float2 (&v)[SmallShape<LG>::E], float2* S0, float2* S1,
+                                           const float2* tw, const OP& op) {
+  using S = SmallShape<LG>;
+  constexpr int N = S::N, R1 = S::E, RL = S::E / 2, M = N / RL, ST1 = N / R1;
+  const int tid = threadIdx.x;
+  const bool act = tid < S::NA;
+  float2 *a = S0, *b = S1;
+  if (act) {
+    dft<R1, -1>(v);
+    float2* q = a + padP(tid * R1);
+#pragma unroll
+    for (int r = 0; r < R1; ++r) q[r] = v[out_slot<R1>(r)];   // padP(tid R1 + r): r stays below the next pad slot
+  }
+  __syncthreads();
+  if constexpr (S::kLgM1 > 0) {
+    small_mid<LG, S::kLg1, S::kLgM1, -1>(a, b, tw + S::kF1);
+    float2* t = a; a = b; b = t;
+  }
+  if constexpr (S::kLgM2 > 0) {
+    small_mid<LG, S::kLg1 + S::kLgM1, S::kLgM2, -1>(a, b, tw + S::kF2);
+    float2* t = a; a = b; b = t;
+  }
+  if (act) {
+    const int j0 = tid, j1 = tid == 0 ? M / 2 : M - tid;
+    float2 x[RL], y[RL];
+    const float2 *q0 = a + padP(j0), *q1 = a + padP(j1);
+#pragma unroll
+    for (int r = 0; r < RL; ++r) {
+      x[r] = q0[padP(r * M)];
+      y[r] = q1[padP(r * M)];
+    }
+    stage_twiddle<RL, -1>(x, tw + S::kFL, M, j0);
+    stage_twiddle<RL, -1>(y, tw + S::kFL, M, j1);
+    dft<RL, -1>(x);
+    dft<RL, -1>(y);
+    float2 p[RL], w[RL];   // frequency order
+#pragma unroll
+    for (int r = 0; r < RL; ++r) {
+      p[r] = x[out_slot<RL>(r)];
+      w[r] = y[out_slot<RL>(r)];
+    }
+    if (tid != 0) {
+#pragma unroll
+      for (int r = 0; r < RL / 2; ++r) {
+        op(j0 + r * M, p[r], w[RL - 1 - r]);
+        op(j1 + r * M, w[r], p[RL - 1 - r]);
+      }
+    } else {
+      float2 z = p[0];
+      op(0, p[0], z);
+#pragma unroll
+      for (int r = 1; r < RL / 2; ++r) op(r * M, p[r], p[RL - r]);
+      z = p[RL / 2];
+      op(N / 2, p[RL / 2], z);
+#pragma unroll
+      for (int r = 0; r < RL / 2; ++r) op(M / 2 + r * M, w[r], w[RL - 1 - r]);
+    }
+    dft<RL, +1>(p);
+    dft<RL, +1>(w);
+    float2 *o0 = b + padP(j0 * RL), *o1 = b + padP(j1 * RL);
+#pragma unroll
+    for (int r = 0; r < RL; ++r) {
+      o0[r] = p[out_slot<RL>(r)];
+      o1[r] = w[out_slot<RL>(r)];
+    }
+  }
+  __syncthreads();
+  { float2* t = a; a = b; b = t; }
+  if constexpr (S::kLgM2 > 0) {
+    small_mid<LG, S::kLgL, S::kLgM2, +1>(a, b, tw + S::kI2);
+    float2* t = a; a = b; b = t;
+  }
+  if constexpr (S::kLgM1 > 0) {
+    small_mid<LG, S::kLgL + S::kLgM2, S::kLgM1, +1>(a, b, tw + S::kI1);
+    float2* t = a; a = b; b = t;
+  }
+  if (act) {
+    const float2* q = a + padP(tid);
+    float2 u[R1];
+#pragma unroll
+    for (int r = 0; r < R1; ++r) u[r] = q[padP(r * ST1)];
+    stage_twiddle<R1, +1>(u, tw + S::kIL, ST1, tid);
+    dft<R1, +1>(u);
+#pragma unroll
+    for (int r = 0; r < R1; ++r) v[r] = u[out_slot<R1>(r)];
+  }
+}
+
+}  // namespace csk
