@@ -297,7 +297,7 @@ cs_status cs_forward_direct(int64_t n, int64_t m, const float* c, const int32_t*
  * owned by another allocator (a framework's caching allocator or a fixed
  * pool), and latency-critical loops that cannot take the device
  * synchronisation an allocation may cause.  No plan is needed and nothing
- * is allocated: the FFT work space is a fixed 768 KiB array inside this
+ * is allocated: the FFT work space is a fixed 256 KiB array inside this
  * library, held on every GPU that loads it until the process exits.
  *   y = C x (transpose = 0) or C^T x (transpose != 0), C[i][j] = c[(j-i) mod n]
  *   n          power of two, 64 <= n <= CS_STATIC_MAX_N (else CS_ERR_UNSUPPORTED)

@@ -436,18 +436,6 @@ cudaError_t launch_tab_admm2d(const double2* chat2, const Geo& g, int64_t n0, in
   return cudaGetLastError();
 }
 
-cudaError_t launch_fft64_complex(double2* a, double2* b, int64_t n, double2** out, cudaStream_t s) {
-  double2* in = a;
-  double2* o = b;
-  for (int64_t Ls = 1; Ls < n; Ls <<= 1) {
-    fft64_stage_k<<<blocks_for(n >> 1), AUX_NT, 0, s>>>(in, o, n, Ls);
-    double2* t = in; in = o; o = t;
-  }
-  *out = in;
-  return cudaGetLastError();
-}
-
-
 cudaError_t launch_tab_ista(const double2* chat, const Geo& g, int64_t n, float4* tabA, cudaStream_t s) {
   const int64_t cnt = tab_count(g);
   tab_ista_k<<<blocks_for(cnt), AUX_NT, 0, s>>>(chat, g, n, tabA, cnt);
