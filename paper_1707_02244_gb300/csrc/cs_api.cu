@@ -635,8 +635,9 @@ cs_status build_plan(cs_plan_t* out, int64_t n0, int64_t n1, int64_t m, const in
       CS_PLAN_TRY(dalloc(&p->sml.tb, n / 2 + 1));
       CS_PLAN_TRY(dalloc(&p->sml.tw_a, small_tw_count(lgn)));
     }
-    CS_PLAN_TRY(launch_small_tables(chat, n, lgn, p->sml.tA, p->sml.tB, p->sml.tc, p->sml.abs2, p->sml.tw_i,
-                                    p->sml.tw_a, s));
+    CS_PLAN_TRY(launch_small_tables(chat, n, p->sml.tA, p->sml.tB, p->sml.tc, p->sml.abs2, s));
+    CS_PLAN_TRY(launch_small_tw(lgn - 1, p->sml.tw_i, s));
+    if (p->small_a) CS_PLAN_TRY(launch_small_tw(lgn, p->sml.tw_a, s));
   }
   CS_PLAN_TRY(admm_table(p, 1.0, 1.0, s, nullptr));
   CS_PLAN_TRY(launch_build_mask(d_rows, m, n, p->gi, 1, p->si.mask, p->status, s));

@@ -1,15 +1,12 @@
 // Batched solver: many independent instances A_i = P_i C(c_i) of uneven size.
 // Every instance with n <= CS_BATCH_MAX_N is solved by one CTA that keeps its
-// iterate in shared memory for all iterations (no global exchange at all: the
-// whole FFT of the instance fits in the CTA); CTAs are ordered largest
-// instance first, one launch per power-of-two size class.  Larger instances
-// have their own plan's buffers and tables but are iterated together: each
-// pass of an iteration is one grouped launch over the tiles of all of them
-// (col_kernel_multi / mid_kernel_multi), so a whole solve of every large
-// instance is one captured CUDA graph on the batch's stream, ordered by the
-// kernel boundaries alone.  Instances whose n is 7-smooth but not a power of
-// two go to the mixed-radix solver of cs_smooth.cu (one persistent launch per
-// solve over all of them).
+// iterate on chip for all iterations (cs_small.cu), one launch per
+// power-of-two size class.  Larger instances have their own plan's buffers
+// and tables but are iterated together: each pass of an iteration is one
+// grouped launch over the tiles of all instances of one length (cs_group.cu),
+// and the lengths run side by side as branches of one captured CUDA graph.
+// Instances whose n is 7-smooth but not a power of two go to the mixed-radix
+// solver of cs_smooth.cu (one persistent launch per solve over all of them).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -27,9 +24,6 @@
 namespace csk {
 namespace {
 
-constexpr int LG_TW = 13;       // master twiddle table exp(-2 pi i q / 8192)
-constexpr int BI_LG_MIN = 5, BI_LG_MAX = 12;   // ISTA: packed length N = n/2 = 2^LG
-constexpr int BA_LG_MIN = 6, BA_LG_MAX = 13;   // ADMM: complex length n = 2^LG
 constexpr int NSIDE_MAX = 4;    // side streams of the size-class launches (within CUDA's default 8 queues)
 
 struct BatchDesc {
@@ -37,260 +31,11 @@ struct BatchDesc {
   int pad0;
   int64_t noff;   // offset of x / z / state in the concatenated n-vectors
   int64_t moff;   // offset of y in the concatenated m-vectors
-  int64_t woff;   // offset of the row-mask words
   int64_t itab;   // ISTA table offset (n/4 + 1 entries)
   int64_t atab;   // ADMM table offset (n/2 + 1 entries)
 };
 
-struct BatchScalars {   // per call
-  float thr, tau, rho, sigma, tau1, tau2, d_on, d_off;
-};
-
-__device__ __forceinline__ float soft(float u, float g) { return u > g ? u - g : (u < -g ? u + g : 0.f); }
-
-// Packed real-FFT spectrum operator of one instance (as in the mid pass,
-// with the pair (k, N - k) of a single vector).
-template <bool ADJ>
-__device__ __forceinline__ void pair_real(const float4 t, float2 be, float2& za, float2& zb) {
-  float2 al = make_float2(t.x, t.y), al2 = make_float2(t.z, t.w);
-  float2 be2 = make_float2(-be.x, be.y);
-  if (!ADJ) {
-    al = cconj(al);
-    al2 = cconj(al2);
-    const float2 tb = be;
-    be = make_float2(-tb.x, tb.y);
-    be2 = tb;
-  }
-  const float2 a2 = za, b2 = zb;
-  za = cadd(cmul(al, a2), cmul(be, cconj(b2)));
-  zb = cadd(cmul(al2, b2), cmul(be2, cconj(a2)));
-}
-
-// One FFT of the instance's vector (length 2^LG, one CTA of 2^LG / 16
-// threads) in shared memory; the shape is fixed at compile time so every
-// address of a stage is a base plus an immediate.
-template <int DIR, int LG>
-__device__ __forceinline__ void fft_vec(float2* S, const float2* __restrict__ tw) {
-  constexpr int L = 1 << LG;
-  const StaticLayout<LG, 0, false> lay;
-  tile_fft<DIR, L, L / EPT>(S, lay, tw, LG_TW);
-}
-
-template <bool ADJ, int N, int NT>
-__device__ __forceinline__ void pair_pass(float2* S, const float4* __restrict__ tA, const float2* __restrict__ tB) {
-  for (int k = threadIdx.x; k <= (N >> 1); k += NT) {
-    const int kp = (N - k) & (N - 1);
-    float2 za = S[pad(k)], zb = S[pad(kp)];
-    pair_real<ADJ>(__ldg(tA + k), __ldg(tB + k), za, zb);
-    S[pad(kp)] = zb;   // self-pairs keep the k-side value
-    S[pad(k)] = za;
-  }
-  __syncthreads();
-}
-
-// One CTA solves instance order[blockIdx.x] (n = 2^(LG+1)) for `iters` ISTA
-// iterations (Algorithm 1, threshold tau * lambda):
-//   x <- eta(x + tau C^T M (y~ - C x)).
-template <int LG>
-__global__ void __launch_bounds__((1 << LG) / EPT) batch_ista_k(
-    const BatchDesc* __restrict__ descs, const BatchScalars* __restrict__ sc, const int* __restrict__ order,
-    const float4* __restrict__ tA, const float2* __restrict__ tB, const uint32_t* __restrict__ mask,
-    const uint32_t* __restrict__ prefix, const float* __restrict__ ys, const float2* __restrict__ tw,
-    float* __restrict__ x, int iters) {
-  constexpr int N = 1 << LG, NT = N / EPT;
-  extern __shared__ float2 sm[];
-  float2* S = sm;
-  float2* X = sm + smem_slots(N);
-  const int id = order[blockIdx.x];
-  const BatchDesc d = descs[id];
-  const BatchScalars s = sc[id];
-  float* xg = x + d.noff;   // 4-byte aligned only: the concatenation may hold odd-length instances
-  const uint32_t* mk = mask + d.woff;
-  const uint32_t* pf = prefix + d.woff;
-  const float* yv = ys + d.moff;
-  const float4* tAi = tA + d.itab;
-  const float2* tBi = tB + d.itab;
-  for (int p = threadIdx.x; p < N; p += NT) {
-    const float2 v = make_float2(xg[2 * p], xg[2 * p + 1]);
-    X[p] = v;
-    S[pad(p)] = v;
-  }
-  __syncthreads();
-#pragma unroll 1
-  for (int it = 0; it < iters; ++it) {
-    fft_vec<-1, LG>(S, tw);
-    pair_pass<false, N, NT>(S, tAi, tBi);
-    fft_vec<+1, LG>(S, tw);
-    // r~ = M (y~ - C x) on rows 2p, 2p+1
-    for (int p = threadIdx.x; p < N; p += NT) {
-      const uint32_t w = mk[p >> 4];
-      const int b = (2 * p) & 31;
-      const int i0 = (int)pf[p >> 4] + __popc(w & ((1u << b) - 1u));
-      const uint32_t mm = (w >> b) & 3u;
-      const float2 v = S[pad(p)];
-      S[pad(p)] = make_float2((mm & 1u) ? yv[i0] - v.x : 0.f, (mm & 2u) ? yv[i0 + (int)(mm & 1u)] - v.y : 0.f);
-    }
-    __syncthreads();
-    fft_vec<-1, LG>(S, tw);
-    pair_pass<true, N, NT>(S, tAi, tBi);
-    fft_vec<+1, LG>(S, tw);
-    for (int p = threadIdx.x; p < N; p += NT) {
-      const float2 g = S[pad(p)], xo = X[p];
-      const float2 xn = make_float2(soft(fmaf(s.tau, g.x, xo.x), s.thr), soft(fmaf(s.tau, g.y, xo.y), s.thr));
-      X[p] = xn;
-      S[pad(p)] = xn;
-    }
-    __syncthreads();
-  }
-  for (int p = threadIdx.x; p < N; p += NT) {
-    xg[2 * p] = X[p].x;
-    xg[2 * p + 1] = X[p].y;
-  }
-}
-
-// One CTA solves instance order[blockIdx.x] (n = 2^LG) for `iters`
-// iterations of Algorithm 3 from the zero state.  The complex-n FFT of
-// (v + mu) + i (z - nu) lives in shared memory; mu and nu in global memory
-// (the instance's slice).
-template <int LG>
-__global__ void __launch_bounds__((1 << LG) / EPT) batch_admm_k(
-    const BatchDesc* __restrict__ descs, const BatchScalars* __restrict__ sc, const int* __restrict__ order,
-    const float2* __restrict__ tc, const float* __restrict__ tb, const uint32_t* __restrict__ mask,
-    const uint32_t* __restrict__ prefix, const float* __restrict__ ys, const float2* __restrict__ tw,
-    float* __restrict__ z, float* __restrict__ mu, float* __restrict__ nu, int iters) {
-  constexpr int n = 1 << LG, NT = n / EPT;
-  extern __shared__ float2 sm[];
-  float2* S = sm;
-  const int id = order[blockIdx.x];
-  const BatchDesc d = descs[id];
-  const BatchScalars s = sc[id];
-  float* zi = z + d.noff;
-  float* mui = mu + d.noff;
-  float* nui = nu + d.noff;
-  const uint32_t* mk = mask + d.woff;
-  const uint32_t* pf = prefix + d.woff;
-  const float* yv = ys + d.moff;
-  const float2* tci = tc + d.atab;
-  const float* tbi = tb + d.atab;
-  for (int p = threadIdx.x; p < n; p += NT) {
-    mui[p] = 0.f;
-    nui[p] = 0.f;
-    S[pad(p)] = make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-#pragma unroll 1
-  for (int it = 0; it < iters; ++it) {
-    fft_vec<-1, LG>(S, tw);
-    // x-update spectrum (Algorithm 3) for every pair (k, n - k):
-    //   V = (Z_k + conj Z_{n-k}) / 2, W = (Z_k - conj Z_{n-k}) / 2i,
-    //   X = bhat (rho chat V + sigma W) / n, then X + i conj(chat) X
-    for (int k = threadIdx.x; k <= (n >> 1); k += NT) {
-      const int kp = (n - k) & (n - 1);
-      const float2 za = S[pad(k)], zb = S[pad(kp)];
-      const float2 ch = __ldg(tci + k);
-      const float bb = __ldg(tbi + k);
-      const float2 V = make_float2(0.5f * (za.x + zb.x), 0.5f * (za.y - zb.y));
-      const float2 Wk = make_float2(0.5f * (za.y + zb.y), -0.5f * (za.x - zb.x));
-      const float2 cv = cmul(ch, V);
-      const float2 X = make_float2(bb * fmaf(s.rho, cv.x, s.sigma * Wk.x), bb * fmaf(s.rho, cv.y, s.sigma * Wk.y));
-      const float2 Pc = cmulc(X, ch);
-      S[pad(kp)] = make_float2(X.x + Pc.y, Pc.x - X.y);
-      S[pad(k)] = make_float2(X.x - Pc.y, X.y + Pc.x);
-    }
-    __syncthreads();
-    fft_vec<+1, LG>(S, tw);
-    const bool last = it == iters - 1;
-    for (int p = threadIdx.x; p < n; p += NT) {
-      const uint32_t w = mk[p >> 5];
-      const int b = p & 31;
-      const bool on = (w >> b) & 1u;
-      const float yvv = on ? yv[pf[p >> 5] + __popc(w & ((1u << b) - 1u))] : 0.f;
-      const float2 xc = S[pad(p)];
-      const float xx = xc.x, cx = xc.y;
-      const float m0 = mui[p], n0 = nui[p];
-      const float vv = (on ? s.d_on : s.d_off) * fmaf(s.rho, cx - m0, yvv);
-      const float zz = soft(xx + n0, s.thr);
-      const float m2 = fmaf(s.tau1, vv - cx, m0);
-      const float n2 = fmaf(s.tau2, xx - zz, n0);
-      mui[p] = m2;
-      nui[p] = n2;
-      if (last) zi[p] = zz;
-      S[pad(p)] = make_float2(vv + m2, zz - n2);
-    }
-    __syncthreads();
-  }
-}
-
-template <int LG>
-size_t ista_smem() { return sizeof(float2) * (smem_slots(1 << LG) + (1 << LG)); }
-template <int LG>
-size_t admm_smem() { return sizeof(float2) * smem_slots(1 << LG); }
-
-// Per size class: the kernel instantiation and its launch shape.
-struct ClassKernel {
-  const void* fn;
-  unsigned nt;
-  size_t smem;
-};
-
-template <int LG>
-ClassKernel ista_kernel() { return {reinterpret_cast<const void*>(&batch_ista_k<LG>), (1u << LG) / EPT, ista_smem<LG>()}; }
-template <int LG>
-ClassKernel admm_kernel() { return {reinterpret_cast<const void*>(&batch_admm_k<LG>), (1u << LG) / EPT, admm_smem<LG>()}; }
-
-ClassKernel ista_class(int lg) {
-  switch (lg) {
-    case 5: return ista_kernel<5>();
-    case 6: return ista_kernel<6>();
-    case 7: return ista_kernel<7>();
-    case 8: return ista_kernel<8>();
-    case 9: return ista_kernel<9>();
-    case 10: return ista_kernel<10>();
-    case 11: return ista_kernel<11>();
-    default: return ista_kernel<12>();
-  }
-}
-
-ClassKernel admm_class(int lg) {
-  switch (lg) {
-    case 6: return admm_kernel<6>();
-    case 7: return admm_kernel<7>();
-    case 8: return admm_kernel<8>();
-    case 9: return admm_kernel<9>();
-    case 10: return admm_kernel<10>();
-    case 11: return admm_kernel<11>();
-    case 12: return admm_kernel<12>();
-    default: return admm_kernel<13>();
-  }
-}
-
 // ---------------------------------------------------------------- plan time
-
-__global__ void tab_ista1_k(const double2* __restrict__ chat, int64_t n, float4* __restrict__ tA,
-                            float2* __restrict__ tB) {
-  // single-vector packed geometry: N = n/2, pairs (k, N - k) for k in [0, N/2]
-  const int64_t N = n >> 1;
-  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (k > (N >> 1)) return;
-  double2 a = chat[k], b = chat[k + N];
-  if (k == 0) { a.y = 0.0; b.y = 0.0; }
-  const double s = 0.5 / (double)N;
-  const double Px = (a.x + b.x) * s, Py = (a.y + b.y) * s, Qx = (a.x - b.x) * s, Qy = (a.y - b.y) * s;
-  double sn, cs;
-  sincospi((double)k / (double)N, &sn, &cs);
-  tA[k] = make_float4((float)(Px - Qx * sn), (float)(Py - Qy * sn), (float)(Px + Qx * sn), (float)(-(Py + Qy * sn)));
-  tB[k] = make_float2((float)(-Qy * cs), (float)(Qx * cs));
-}
-
-__global__ void tab_admm1_k(const double2* __restrict__ chat, int64_t n, float2* __restrict__ tc,
-                            double* __restrict__ abs2) {
-  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (k > (n >> 1)) return;
-  double2 a = chat[k];
-  if (k == 0 || k == (n >> 1)) a.y = 0.0;
-  tc[k] = make_float2((float)a.x, (float)a.y);
-  abs2[k] = a.x * a.x + a.y * a.y;
-}
 
 __global__ void tab_admm1_b_k(const double* __restrict__ abs2, int64_t count, const int* __restrict__ inst,
                               const BatchDesc* __restrict__ descs, const double* __restrict__ rho,
@@ -301,35 +46,16 @@ __global__ void tab_admm1_b_k(const double* __restrict__ abs2, int64_t count, co
   tb[t] = (float)(1.0 / ((double)descs[i].n * (rho[i] * abs2[t] + sigma[i])));
 }
 
-__global__ void batch_mask_k(const int64_t* __restrict__ rows, int64_t m, int64_t n, uint32_t* mask,
-                             int* status) {
+// rows of one instance as int32, range and repeats checked (mask: n bits, zero)
+__global__ void batch_rows_k(const int64_t* __restrict__ rows, int64_t m, int64_t n, uint32_t* mask,
+                             int32_t* __restrict__ rows32, int* status) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= m) return;
   const int64_t r = rows[i];
   if (r < 0 || r >= n) { atomicOr(status, STS_BAD_ROW); return; }
   const uint32_t bit = 1u << (r & 31);
   if (atomicOr(mask + (r >> 5), bit) & bit) atomicOr(status, STS_DUP_ROW);
-}
-
-__global__ void batch_pos_k(const int64_t* __restrict__ rows, int64_t m, const uint32_t* __restrict__ mask,
-                            const uint32_t* __restrict__ prefix, int64_t moff, int32_t* __restrict__ pos) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= m) return;
-  const int64_t r = rows[i];
-  const uint32_t w = mask[r >> 5];
-  pos[i] = (int32_t)(moff + prefix[r >> 5] + __popc(w & ((1u << (r & 31)) - 1u)));
-}
-
-// pos < 0 marks measurements of instances solved by their own plan
-__global__ void batch_scatter_k(const float* __restrict__ y, const int32_t* __restrict__ pos, int64_t count,
-                                float* __restrict__ ys, int* status) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= count) return;
-  const int32_t q = pos[i];
-  if (q < 0) return;
-  const float v = y[i];
-  if (!isfinite(v)) atomicOr(status, STS_NONFINITE);
-  ys[q] = v;
+  rows32[i] = (int32_t)r;
 }
 
 inline unsigned nb256(int64_t c) { return (unsigned)((c + 255) / 256); }
@@ -348,16 +74,24 @@ struct cs_batch_s {
   std::vector<int> smooth_ids;      // 7-smooth, not power-of-two n: the mixed-radix solver
   SmoothSet* smooth = nullptr;
   std::vector<cs_plan_t> plans;     // per large instance
-  // grouped launches over the large instances (in the order of `large`)
+  // grouped launches over the large instances (in the order of `large`,
+  // which is by length): one chain of passes per length
+  struct Chain {
+    Geo gi, ga;
+    int col_i0, n_col_i, mid_i0, n_mid_i, col_a0, n_col_a, mid_a0, n_mid_a;   // ranges of the maps
+    cudaStream_t cap;             // capture-only stream of this chain (the first uses Group::cap)
+    cudaEvent_t done;
+  };
   struct Group {
     int count = 0;
     std::vector<GroupDesc> hdesc;
+    std::vector<Chain> chains;
     GroupDesc* desc = nullptr;
     KParams *kps_i = nullptr, *kps_a0 = nullptr, *kps_a1 = nullptr;
     CallArgs* ca = nullptr;
     int2 *map_col_i = nullptr, *map_mid_i = nullptr, *map_col_a = nullptr, *map_mid_a = nullptr;
-    int n_col_i = 0, n_mid_i = 0, n_col_a = 0, n_mid_a = 0;
     cudaStream_t cap = nullptr;
+    cudaEvent_t fork = nullptr;
     std::map<uint64_t, cudaGraphExec_t> graphs;
   } grp;
   struct Class {
@@ -369,8 +103,8 @@ struct cs_batch_s {
   cudaEvent_t side_done[NSIDE_MAX] = {};
   cudaEvent_t fork = nullptr;
   BatchDesc* descs = nullptr;
-  BatchScalars* sc = nullptr;
-  int* order = nullptr;
+  SmallInst* insts = nullptr;       // in the order of `small`
+  SmallScalars* sc = nullptr;
   float4* tA = nullptr;
   float2* tB = nullptr;
   float2* tc = nullptr;
@@ -379,12 +113,8 @@ struct cs_batch_s {
   int* tb_inst = nullptr;           // instance of every ADMM table entry
   double* drho = nullptr;
   double* dsigma = nullptr;
-  uint32_t* mask = nullptr;
-  uint32_t* prefix = nullptr;
-  int32_t* pos = nullptr;
-  float* ys = nullptr;
-  float2* tw = nullptr;
-  float *amu = nullptr, *anu = nullptr;
+  int32_t* rows32 = nullptr;
+  float2* tw = nullptr;             // stage twiddles of every transform length in use
   int* status = nullptr;
   int64_t ntot = 0, mtot = 0, atab_tot = 0;
   std::vector<double> host_rho, host_sigma;
@@ -397,8 +127,8 @@ void batch_free(cs_batch_s* b) {
   for (cs_plan_t p : b->plans)
     if (p) cs_plan_destroy(p);
   smooth_free(b->smooth);
-  void* bufs[] = {b->descs, b->sc,   b->order,  b->tA,  b->tB, b->tc, b->abs2, b->tb,  b->tb_inst,
-                  b->drho,  b->dsigma, b->mask, b->prefix, b->pos, b->ys, b->tw, b->amu, b->anu, b->status};
+  void* bufs[] = {b->descs, b->insts, b->sc,     b->tA,     b->tB, b->tc,   b->abs2,
+                  b->tb,    b->tb_inst, b->drho, b->dsigma, b->rows32, b->tw, b->status};
   for (void* q : bufs)
     if (q) cudaFree(q);
   for (int k = 0; k < NSIDE_MAX; ++k) {
@@ -411,6 +141,11 @@ void batch_free(cs_batch_s* b) {
   void* gb[] = {G.desc, G.kps_i, G.kps_a0, G.kps_a1, G.ca, G.map_col_i, G.map_mid_i, G.map_col_a, G.map_mid_a};
   for (void* q : gb)
     if (q) cudaFree(q);
+  for (auto& ch : G.chains) {
+    if (ch.cap && ch.cap != G.cap) cudaStreamDestroy(ch.cap);
+    if (ch.done) cudaEventDestroy(ch.done);
+  }
+  if (G.fork) cudaEventDestroy(G.fork);
   if (G.cap) cudaStreamDestroy(G.cap);
   delete b;
 }
@@ -473,35 +208,51 @@ cudaError_t run_group_graph(cs_batch_s* b, uint64_t key, F&& enqueue) {
   return cudaGraphLaunch(it->second, b->stream);
 }
 
-// T iterations of Algorithm 1 on every large instance: per iteration four
-// grouped passes (C x, residual, C^T r, update), each over the tiles of all
-// of them.
-cudaError_t enqueue_group_ista(cs_batch_s* b, int T, cudaStream_t s) {
-  auto& G = b->grp;
-  cudaError_t e = launch_col_multi(COL_LOAD, G.kps_i, G.map_col_i, G.n_col_i, s);
+// T iterations of Algorithm 1 on the instances of one length: per iteration
+// four grouped passes (C x, residual, C^T r, update).
+cudaError_t enqueue_chain_ista(const cs_batch_s::Group& G, const cs_batch_s::Chain& c, int T, cudaStream_t s) {
+  auto col = [&](ColKind k) { return launch_col_multi(k, c.gi, G.kps_i, G.map_col_i + c.col_i0, c.n_col_i, s); };
+  auto mid = [&](MidKind k) { return launch_mid_multi(k, c.gi, G.kps_i, G.map_mid_i + c.mid_i0, c.n_mid_i, s); };
+  cudaError_t e = col(COL_LOAD);
   for (int t = 0; t < T && e == cudaSuccess; ++t) {
-    e = launch_mid_multi(MID_FWD, G.kps_i, G.map_mid_i, G.n_mid_i, s);
-    if (e == cudaSuccess) e = launch_col_multi(COL_RESIDUAL, G.kps_i, G.map_col_i, G.n_col_i, s);
-    if (e == cudaSuccess) e = launch_mid_multi(MID_ADJ, G.kps_i, G.map_mid_i, G.n_mid_i, s);
-    if (e == cudaSuccess)
-      e = launch_col_multi(t + 1 < T ? COL_ISTA : COL_ISTA_LAST, G.kps_i, G.map_col_i, G.n_col_i, s);
+    e = mid(MID_FWD);
+    if (e == cudaSuccess) e = col(COL_RESIDUAL);
+    if (e == cudaSuccess) e = mid(MID_ADJ);
+    if (e == cudaSuccess) e = col(t + 1 < T ? COL_ISTA : COL_ISTA_LAST);
   }
   return e;
 }
 
-// T iterations of Algorithm 3 on every large instance: per iteration the
-// grouped x-update (mid pass) and elementwise steps (column pass); the last
-// one writes z.
-cudaError_t enqueue_group_admm(cs_batch_s* b, int T, cudaStream_t s) {
-  auto& G = b->grp;
-  cudaError_t e = launch_col_multi(COL_ADMM_INIT, G.kps_a0, G.map_col_a, G.n_col_a, s);
+// T iterations of Algorithm 3 on the instances of one length: per iteration
+// the grouped x-update (mid pass) and elementwise steps (column pass); the
+// last one writes z.
+cudaError_t enqueue_chain_admm(const cs_batch_s::Group& G, const cs_batch_s::Chain& c, int T, cudaStream_t s) {
+  auto col = [&](ColKind k, const KParams* kps) {
+    return launch_col_multi(k, c.ga, kps, G.map_col_a + c.col_a0, c.n_col_a, s);
+  };
+  cudaError_t e = col(COL_ADMM_INIT, G.kps_a0);
   for (int t = 0; t < T && e == cudaSuccess; ++t) {
-    e = launch_mid_multi(MID_ADMM, G.kps_a0, G.map_mid_a, G.n_mid_a, s);
-    if (e == cudaSuccess) {
-      const bool last = t + 1 == T;
-      e = launch_col_multi(last ? COL_ADMM_LAST : COL_ADMM, last ? G.kps_a1 : G.kps_a0,
-                           G.map_col_a, G.n_col_a, s);
-    }
+    e = launch_mid_multi(MID_ADMM, c.ga, G.kps_a0, G.map_mid_a + c.mid_a0, c.n_mid_a, s);
+    const bool last = t + 1 == T;
+    if (e == cudaSuccess) e = col(last ? COL_ADMM_LAST : COL_ADMM, last ? G.kps_a1 : G.kps_a0);
+  }
+  return e;
+}
+
+// Every length's chain as a branch of the captured graph, forked from `s` and
+// joined back.  Lengths are independent, and a chain's passes only fill the
+// chip where it has many instances: side by side they fill each other's
+// partial waves, and a short length does not wait for a long one's passes.
+template <class F>
+cudaError_t enqueue_chains(cs_batch_s* b, cudaStream_t s, F&& chain) {
+  auto& G = b->grp;
+  cudaError_t e = cudaEventRecord(G.fork, s);
+  for (auto& c : G.chains) {
+    if (e == cudaSuccess && c.cap != s) e = cudaStreamWaitEvent(c.cap, G.fork, 0);
+    if (e == cudaSuccess) e = chain(c, c.cap);
+    if (c.cap == s) continue;
+    if (e == cudaSuccess) e = cudaEventRecord(c.done, c.cap);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, c.done, 0);
   }
   return e;
 }
@@ -530,7 +281,7 @@ cs_status cs_batch_plan(cs_batch_t* out, int count, const int64_t* n, const int6
   b->noff.resize(count);
   b->moff.resize(count);
   std::vector<BatchDesc> hd(count);
-  int64_t no = 0, mo = 0, wo = 0, it = 0, at = 0;
+  int64_t no = 0, mo = 0, it = 0, at = 0;
   for (int i = 0; i < count; ++i) {
     b->noff[i] = no;
     b->moff[i] = mo;
@@ -541,7 +292,6 @@ cs_status cs_batch_plan(cs_batch_t* out, int count, const int64_t* n, const int6
     d.pad0 = 0;
     d.noff = no;
     d.moff = mo;
-    d.woff = wo;
     d.itab = it;
     d.atab = at;
     no += n[i];
@@ -550,7 +300,6 @@ cs_status cs_batch_plan(cs_batch_t* out, int count, const int64_t* n, const int6
       b->smooth_ids.push_back(i);
     } else if (n[i] <= CS_BATCH_MAX_N) {
       b->small.push_back(i);
-      wo += n[i] / 32;
       it += n[i] / 4 + 1;
       at += n[i] / 2 + 1;
     } else {
@@ -615,9 +364,8 @@ cs_status cs_batch_plan(cs_batch_t* out, int count, const int64_t* n, const int6
   if (!b->large.empty()) {
     auto& G = b->grp;
     G.count = (int)b->large.size();
-    CS_B_TRY(init_col_multi_kernels());
-    CS_B_TRY(init_mid_multi_kernels());
     CS_B_TRY(cudaStreamCreateWithFlags(&G.cap, cudaStreamNonBlocking));
+    CS_B_TRY(cudaEventCreateWithFlags(&G.fork, cudaEventDisableTiming));
     CS_B_TRY(balloc(&G.desc, G.count));
     CS_B_TRY(balloc(&G.kps_i, G.count));
     CS_B_TRY(balloc(&G.kps_a0, G.count));
@@ -637,18 +385,36 @@ cs_status cs_batch_plan(cs_batch_t* out, int count, const int64_t* n, const int6
       ki[j].ca = ka0[j].ca = G.ca + j;
       ka1[j] = ka0[j];
       ka1[j].flags = FL_WRITE_STATE;
+      // grouped launches take 4096-value tiles of a fixed set of shapes
+      if (j == 0 || n[i] != n[b->large[j - 1]]) {
+        cs_batch_s::Chain ch{};
+        ch.gi = d.gi;
+        ch.ga = d.ga;
+        ch.col_i0 = (int)mci.size();
+        ch.mid_i0 = (int)mmi.size();
+        ch.col_a0 = (int)mca.size();
+        ch.mid_a0 = (int)mma.size();
+        G.chains.push_back(ch);
+        auto& c = G.chains.back();
+        if (G.chains.size() == 1) c.cap = G.cap;
+        else CS_B_TRY(cudaStreamCreateWithFlags(&c.cap, cudaStreamNonBlocking));
+        CS_B_TRY(cudaEventCreateWithFlags(&c.done, cudaEventDisableTiming));
+        for (const Geo* g : {&d.gi, &d.ga}) {
+          const cudaError_t eg = init_multi_kernels(*g);
+          if (eg == cudaErrorInvalidValue) return fail(CS_ERR_UNSUPPORTED);
+          CS_B_TRY(eg);
+        }
+      }
+      auto& ch = G.chains.back();
+      ch.n_col_i += d.gi.col_ctas;
+      ch.n_mid_i += d.gi.mid_ctas;
+      ch.n_col_a += d.ga.col_ctas;
+      ch.n_mid_a += d.ga.mid_ctas;
       for (int t = 0; t < d.gi.col_ctas; ++t) mci.push_back(make_int2(j, t));
       for (int t = 0; t < d.gi.mid_ctas; ++t) mmi.push_back(make_int2(j, t));
       for (int t = 0; t < d.ga.col_ctas; ++t) mca.push_back(make_int2(j, t));
       for (int t = 0; t < d.ga.mid_ctas; ++t) mma.push_back(make_int2(j, t));
-      // grouped launches take 4096-value tiles and run-time shapes only
-      if (d.gi.tile != 4096 || d.ga.tile != 4096 || d.gi.col_tile != 4096 || d.ga.col_tile != 4096)
-        return fail(CS_ERR_UNSUPPORTED);
     }
-    G.n_col_i = (int)mci.size();
-    G.n_mid_i = (int)mmi.size();
-    G.n_col_a = (int)mca.size();
-    G.n_mid_a = (int)mma.size();
     CS_B_TRY(balloc(&G.map_col_i, mci.size()));
     CS_B_TRY(balloc(&G.map_mid_i, mmi.size()));
     CS_B_TRY(balloc(&G.map_col_a, mca.size()));
@@ -664,17 +430,18 @@ cs_status cs_batch_plan(cs_batch_t* out, int count, const int64_t* n, const int6
     CS_B_TRY(cudaStreamSynchronize(s));
   }
   if (!b->small.empty()) {
-    for (int lg = BI_LG_MIN; lg <= BI_LG_MAX; ++lg) {
-      const ClassKernel k = ista_class(lg);
-      CS_B_TRY(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem));
-    }
-    for (int lg = BA_LG_MIN; lg <= BA_LG_MAX; ++lg) {
-      const ClassKernel k = admm_class(lg);
-      CS_B_TRY(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem));
-    }
+    // stage twiddles of the lengths in use (ISTA 2^(lgn-1), ADMM 2^lgn)
+    std::map<int, int64_t> twoff;
+    int64_t twn = 0;
+    for (int i : b->small)
+      for (int lg : {hd[i].lgn - 1, hd[i].lgn})
+        if (twoff.emplace(lg, twn).second) twn += (small_tw_count(lg) + 1) & ~1;
+    const int ns = (int)b->small.size();
+    int64_t ms = 0;
+    for (int i : b->small) ms += m[i];
     CS_B_TRY(balloc(&b->descs, count));
+    CS_B_TRY(balloc(&b->insts, ns));
     CS_B_TRY(balloc(&b->sc, count));
-    CS_B_TRY(balloc(&b->order, b->small.size()));
     CS_B_TRY(balloc(&b->tA, it));
     CS_B_TRY(balloc(&b->tB, it));
     CS_B_TRY(balloc(&b->tc, at));
@@ -683,20 +450,33 @@ cs_status cs_batch_plan(cs_batch_t* out, int count, const int64_t* n, const int6
     CS_B_TRY(balloc(&b->tb_inst, at));
     CS_B_TRY(balloc(&b->drho, count));
     CS_B_TRY(balloc(&b->dsigma, count));
-    CS_B_TRY(balloc(&b->mask, wo));
-    CS_B_TRY(balloc(&b->prefix, wo));
-    CS_B_TRY(balloc(&b->pos, mo));
-    CS_B_TRY(balloc(&b->ys, mo));
-    CS_B_TRY(balloc(&b->tw, 1 << LG_TW));
-    CS_B_TRY(balloc(&b->amu, no));
-    CS_B_TRY(balloc(&b->anu, no));
+    CS_B_TRY(balloc(&b->rows32, ms));
+    CS_B_TRY(balloc(&b->tw, twn));
     CS_B_TRY(balloc(&b->status, 1));
     CS_B_TRY(cudaMemsetAsync(b->status, 0, sizeof(int), s));
-    CS_B_TRY(cudaMemsetAsync(b->mask, 0, (wo ? wo : 1) * sizeof(uint32_t), s));
-    CS_B_TRY(cudaMemsetAsync(b->pos, 0xff, (mo ? mo : 1) * sizeof(int32_t), s));   // -1: not a small instance
     CS_B_TRY(cudaMemcpyAsync(b->descs, hd.data(), count * sizeof(BatchDesc), cudaMemcpyHostToDevice, s));
-    CS_B_TRY(cudaMemcpyAsync(b->order, b->small.data(), b->small.size() * sizeof(int), cudaMemcpyHostToDevice, s));
-    CS_B_TRY(launch_twiddle(b->tw, 1 << LG_TW, 1 << LG_TW, s));
+    for (const auto& kv : twoff) CS_B_TRY(launch_small_tw(kv.first, b->tw + kv.second, s));
+    std::vector<SmallInst> hs_inst(ns);
+    ms = 0;
+    for (int k = 0; k < ns; ++k) {
+      const BatchDesc& d = hd[b->small[k]];
+      SmallInst& q = hs_inst[k];
+      q = SmallInst{};
+      q.tA = b->tA + d.itab;
+      q.tB = b->tB + d.itab;
+      q.tc = b->tc + d.atab;
+      q.tb = b->tb + d.atab;
+      q.tw_i = b->tw + twoff[d.lgn - 1];
+      q.tw_a = b->tw + twoff[d.lgn];
+      q.rows = b->rows32 + ms;
+      q.status = b->status;
+      q.noff = d.noff;
+      q.moff = d.moff;
+      q.m = d.m;
+      q.id = b->small[k];
+      ms += d.m;
+    }
+    CS_B_TRY(cudaMemcpyAsync(b->insts, hs_inst.data(), ns * sizeof(SmallInst), cudaMemcpyHostToDevice, s));
     std::vector<int> inst(at);
     int64_t nmax = 0, mmax = 0;
     for (int i : b->small) {
@@ -708,31 +488,32 @@ cs_status cs_batch_plan(cs_batch_t* out, int count, const int64_t* n, const int6
     double* dc = nullptr;
     double2 *fa = nullptr, *fb = nullptr;
     int64_t* drows = nullptr;
+    uint32_t* dmask = nullptr;
+    CS_B_TRY(balloc(&dmask, nmax / 32));
     CS_B_TRY(balloc(&dc, nmax));
     CS_B_TRY(balloc(&fa, nmax));
     CS_B_TRY(balloc(&fb, nmax));
     CS_B_TRY(balloc(&drows, mmax));
     cudaError_t e = cudaSuccess;
-    for (int i : b->small) {
+    for (int k = 0; k < ns; ++k) {
+      const int i = b->small[k];
       const BatchDesc& d = hd[i];
       if (e == cudaSuccess) e = cudaMemcpyAsync(dc, c + d.noff, n[i] * sizeof(double), cudaMemcpyHostToDevice, s);
       if (e == cudaSuccess) e = cudaMemcpyAsync(drows, rows + d.moff, m[i] * sizeof(int64_t), cudaMemcpyHostToDevice, s);
+      if (e == cudaSuccess) e = cudaMemsetAsync(dmask, 0, n[i] / 32 * sizeof(uint32_t), s);
       double2* chat = nullptr;
       if (e == cudaSuccess) e = launch_fft64(dc, fa, fb, n[i], &chat, s);
+      if (e == cudaSuccess)
+        e = launch_small_tables(chat, n[i], b->tA + d.itab, b->tB + d.itab, b->tc + d.atab, b->abs2 + d.atab, s);
       if (e == cudaSuccess) {
-        tab_ista1_k<<<nb256(n[i] / 4 + 1), 256, 0, s>>>(chat, n[i], b->tA + d.itab, b->tB + d.itab);
-        tab_admm1_k<<<nb256(n[i] / 2 + 1), 256, 0, s>>>(chat, n[i], b->tc + d.atab, b->abs2 + d.atab);
-        batch_mask_k<<<nb256(m[i]), 256, 0, s>>>(drows, m[i], n[i], b->mask + d.woff, b->status);
-        e = launch_prefix(b->mask + d.woff, n[i] / 32, b->prefix + d.woff, s);
-      }
-      if (e == cudaSuccess) {
-        batch_pos_k<<<nb256(m[i]), 256, 0, s>>>(drows, m[i], b->mask + d.woff, b->prefix + d.woff, d.moff,
-                                                 b->pos + d.moff);
+        batch_rows_k<<<nb256(m[i]), 256, 0, s>>>(drows, m[i], n[i], dmask, const_cast<int32_t*>(hs_inst[k].rows),
+                                                  b->status);
         e = cudaGetLastError();
       }
       // the staging buffers are reused by the next instance: keep the order
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     }
+    cudaFree(dmask);
     cudaFree(dc);
     cudaFree(fa);
     cudaFree(fb);
@@ -775,16 +556,15 @@ cs_status cs_batch_ista(cs_batch_t b, const float* y, const float* lambda, const
     if (!(lambda[i] >= 0.f) || !(tau[i] > 0.f) || !std::isfinite(lambda[i]) || !std::isfinite(tau[i])) return CS_ERR_ARG;
   cudaStream_t s = b->stream;
   if (!b->small.empty() && iters > 0) {
-    std::vector<BatchScalars> h(b->count);
+    std::vector<SmallScalars> h(b->count);
     for (int i = 0; i < b->count; ++i) {
-      h[i] = BatchScalars{};
+      h[i] = SmallScalars{};
       h[i].thr = (float)((double)tau[i] * (double)lambda[i]);
       h[i].tau = tau[i];
     }
-    const cs_status st = cstat(cudaMemcpyAsync(b->sc, h.data(), b->count * sizeof(BatchScalars),
+    const cs_status st = cstat(cudaMemcpyAsync(b->sc, h.data(), b->count * sizeof(SmallScalars),
                                                cudaMemcpyHostToDevice, s));
     if (st != CS_OK) return st;
-    batch_scatter_k<<<nb256(b->mtot), 256, 0, s>>>(y, b->pos, b->mtot, b->ys, b->status);
   }
   cs_status st = cstat(fork_sides(b));
   if (!b->large.empty() && st == CS_OK) {
@@ -804,18 +584,19 @@ cs_status cs_batch_ista(cs_batch_t b, const float* y, const float* lambda, const
       st = cstat(launch_group_ista_in(G.desc, G.count, x, s));
       if (st == CS_OK)
         st = cstat(run_group_graph(b, (uint64_t(1) << 40) | (uint32_t)iters,
-                                   [&](cudaStream_t cs) { return enqueue_group_ista(b, iters, cs); }));
+                                   [&](cudaStream_t cs) {
+                                     return enqueue_chains(b, cs, [&](const cs_batch_s::Chain& c, cudaStream_t t) {
+                                       return enqueue_chain_ista(G, c, iters, t);
+                                     });
+                                   }));
       if (st == CS_OK) st = cstat(launch_group_ista_out(G.desc, G.count, x, s));
     }
   }
   if (iters > 0) {
     for (const auto& cl : b->classes) {
       if (st != CS_OK) break;
-      const ClassKernel k = ista_class(cl.lgn - 1);
-      const int* ord = b->order + cl.start;
-      void* args[] = {&b->descs, &b->sc, (void*)&ord, &b->tA, &b->tB, &b->mask, &b->prefix, &b->ys, &b->tw,
-                      (void*)&x, (void*)&iters};
-      st = cstat(cudaLaunchKernel(k.fn, dim3((unsigned)cl.count), dim3(k.nt), args, k.smem, b->side[cl.side]));
+      st = cstat(launch_small_class(false, cl.lgn - 1, b->insts + cl.start, cl.count, b->sc, y, x, iters,
+                                    b->side[cl.side]));
     }
   }
   const cs_status sj = cstat(join_sides(b));
@@ -838,13 +619,13 @@ cs_status cs_batch_admm(cs_batch_t b, const float* y, const float* lambda, const
   if (!b->small.empty() && iters > 0) {
     // sigma = rho, tau1 = tau2 = 1 (as cs_admm); B's spectrum re-tabulated when rho changes
     bool changed = false;
-    std::vector<BatchScalars> h(b->count);
+    std::vector<SmallScalars> h(b->count);
     for (int i = 0; i < b->count; ++i) {
       const double r = rho[i];
       if (r != b->host_rho[i]) changed = true;
       b->host_rho[i] = r;
       b->host_sigma[i] = r;
-      h[i] = BatchScalars{};
+      h[i] = SmallScalars{};
       h[i].thr = (float)((double)lambda[i] / r);
       h[i].rho = (float)r;
       h[i].sigma = (float)r;
@@ -853,7 +634,7 @@ cs_status cs_batch_admm(cs_batch_t b, const float* y, const float* lambda, const
       h[i].d_on = (float)(1.0 / (1.0 + r));
       h[i].d_off = (float)(1.0 / r);
     }
-    st = cstat(cudaMemcpyAsync(b->sc, h.data(), b->count * sizeof(BatchScalars), cudaMemcpyHostToDevice, s));
+    st = cstat(cudaMemcpyAsync(b->sc, h.data(), b->count * sizeof(SmallScalars), cudaMemcpyHostToDevice, s));
     if (st != CS_OK) return st;
     if (changed) {
       st = cstat(cudaMemcpyAsync(b->drho, b->host_rho.data(), b->count * sizeof(double), cudaMemcpyHostToDevice, s));
@@ -864,7 +645,6 @@ cs_status cs_batch_admm(cs_batch_t b, const float* y, const float* lambda, const
       tab_admm1_b_k<<<nb256(b->atab_tot), 256, 0, s>>>(b->abs2, b->atab_tot, b->tb_inst, b->descs, b->drho,
                                                         b->dsigma, b->tb);
     }
-    batch_scatter_k<<<nb256(b->mtot), 256, 0, s>>>(y, b->pos, b->mtot, b->ys, b->status);
   }
   st = cstat(fork_sides(b));
   if (!b->large.empty() && st == CS_OK) {
@@ -893,17 +673,18 @@ cs_status cs_batch_admm(cs_batch_t b, const float* y, const float* lambda, const
     if (st == CS_OK) st = cstat(launch_group_scatter_y(G.desc, G.count, y, 1, b->status, s));
     if (st == CS_OK && iters > 0)
       st = cstat(run_group_graph(b, (uint64_t(2) << 40) | (uint32_t)iters,
-                                 [&](cudaStream_t cs) { return enqueue_group_admm(b, iters, cs); }));
+                                 [&](cudaStream_t cs) {
+                                   return enqueue_chains(b, cs, [&](const cs_batch_s::Chain& c, cudaStream_t t) {
+                                     return enqueue_chain_admm(G, c, iters, t);
+                                   });
+                                 }));
     if (st == CS_OK) st = cstat(launch_group_admm_out(G.desc, G.count, z, s));
   }
   if (iters > 0) {
     for (const auto& cl : b->classes) {
       if (st != CS_OK) break;
-      const ClassKernel k = admm_class(cl.lgn);
-      const int* ord = b->order + cl.start;
-      void* args[] = {&b->descs, &b->sc, (void*)&ord, &b->tc, &b->tb, &b->mask, &b->prefix, &b->ys, &b->tw,
-                      (void*)&z, &b->amu, &b->anu, (void*)&iters};
-      st = cstat(cudaLaunchKernel(k.fn, dim3((unsigned)cl.count), dim3(k.nt), args, k.smem, b->side[cl.side]));
+      st = cstat(launch_small_class(true, cl.lgn, b->insts + cl.start, cl.count, b->sc, y, z, iters,
+                                    b->side[cl.side]));
     }
   }
   const cs_status sj = cstat(join_sides(b));

@@ -59,10 +59,13 @@ struct EpiHook {
 // G = 4 columns, the geometry of every N >= 2^20, fixed at compile time.
 // SHAPE 10 + LGN2 (LGN2 = 5 .. 9): radix-8 tiles of 4 columns (8 for
 // LGN2 = 5), 8 values per thread.
+// SHAPE 40 + LGN2 (LGN2 = 6 .. 9): 4096-value tiles, 16 values per thread
+// (grouped launches).
 template <int SHAPE> struct ColShape {
-  static_assert(SHAPE >= 15 && SHAPE <= 19, "radix-8 column shapes");
-  static constexpr int kLgN2 = SHAPE - 10, kLgG = kLgN2 == 5 ? 3 : 2;
-  using Lay = StaticLayout<kLgN2, kLgG, true, 3>;
+  static_assert((SHAPE >= 15 && SHAPE <= 19) || (SHAPE >= 46 && SHAPE <= 49), "column shapes");
+  static constexpr bool kR8 = SHAPE < 40;
+  static constexpr int kLgN2 = SHAPE % (kR8 ? 10 : 40), kLgG = kR8 ? (kLgN2 == 5 ? 3 : 2) : 12 - kLgN2;
+  using Lay = StaticLayout<kLgN2, kLgG, true, kR8 ? 3 : 4>;
   __device__ static Lay lay(const Geo&) { return Lay{}; }
   __device__ static constexpr int lgG(const Geo&) { return kLgG; }
   __device__ static constexpr int lgN2(const Geo&) { return kLgN2; }
@@ -103,9 +106,9 @@ struct ColIO {
 };
 
 template <int SHAPE> struct ColTile {
-  static constexpr bool kR8 = SHAPE >= 10;
+  static constexpr bool kR8 = SHAPE >= 10 && SHAPE < 40;
   static constexpr int kVpt = kR8 ? VPT8 : EPT;
-  static constexpr int kLgN2 = kR8 ? SHAPE - 10 : SHAPE == 3 ? 12 : 10;   // static shapes
+  static constexpr int kLgN2 = kR8 ? SHAPE - 10 : SHAPE > 40 ? SHAPE - 40 : SHAPE == 3 ? 12 : 10;   // static shapes
   static constexpr int kTile = kR8 ? (kLgN2 == 5 ? 256 : 4 << kLgN2) : SHAPE == 3 ? COL_TILE4 : COL_TILE;
   static constexpr int kMinB = kR8 ? Cfg<kTile, kVpt>::MINB : SHAPE == 3 ? COL_MINB4 : COL_MINB;
   static constexpr int kCarve = kR8 ? 0 : kMinB;

@@ -134,13 +134,14 @@ size_t pass_smem_bytes(int tile);
 // Shared-memory attributes of the pass kernels that geometry g launches.
 cudaError_t init_col_kernels(const Geo& g);
 cudaError_t init_mid_kernels(const Geo& g);
-// Grouped launches over many plans (batched solves, run-time shapes,
-// 4096-value tiles): CTA b runs tile map[b].y of the plan whose parameters
-// are kps[map[b].x] (both device arrays).
-cudaError_t launch_col_multi(ColKind kind, const KParams* kps, const int2* map, int nctas, cudaStream_t s);
-cudaError_t launch_mid_multi(MidKind kind, const KParams* kps, const int2* map, int nctas, cudaStream_t s);
-cudaError_t init_col_multi_kernels();
-cudaError_t init_mid_multi_kernels();
+// Grouped launches over many plans of one length (batched solves, cs_group.cu;
+// 4096-value tiles): CTA b runs tile map[b].y of the plan whose parameters are
+// kps[map[b].x] (both device arrays), g their common geometry.
+cudaError_t launch_col_multi(ColKind kind, const Geo& g, const KParams* kps, const int2* map, int nctas,
+                             cudaStream_t s);
+cudaError_t launch_mid_multi(MidKind kind, const Geo& g, const KParams* kps, const int2* map, int nctas,
+                             cudaStream_t s);
+cudaError_t init_multi_kernels(const Geo& g);
 
 // Small kernels (cs_aux.cu).
 cudaError_t launch_set_args(const CallArgs& a, CallArgs* dst, cudaStream_t s);
@@ -148,9 +149,6 @@ cudaError_t launch_finalize(const double* partials, int nblk, double* stats, cud
 cudaError_t launch_twiddle(float2* dst, int count, int64_t M, cudaStream_t s);
 cudaError_t launch_fft64(const double* c, double2* a, double2* b, int64_t n, double2** out,
                          cudaStream_t s);
-// Forward FP64 FFT of the complex vector in a (b is work space); *out is
-// whichever of a / b holds the result.
-cudaError_t launch_fft64_complex(double2* a, double2* b, int64_t n, double2** out, cudaStream_t s);
 cudaError_t launch_tab_ista(const double2* chat, const Geo& g, int64_t n, float4* tabA, cudaStream_t s);
 // 2D: chat2 is the n0 x n1 FP64 spectrum (row-major); g the 2D geometry.
 cudaError_t launch_tab_ista2d(const double2* chat2, const Geo& g, int64_t n0, int64_t n1, float4* tabA,
@@ -218,9 +216,29 @@ struct SmallArgs {
 };
 cudaError_t launch_small(SmallKind kind, int lgN, const SmallArgs& a, cudaStream_t s);
 int small_tw_count(int lgN);
-// Tables of a plan of n = 2^lgn from its FP64 spectrum (tc, abs2, tw_a null: no ADMM).
-cudaError_t launch_small_tables(const double2* chat, int64_t n, int lgn, float4* tA, float2* tB, float2* tc,
-                                double* abs2, float2* tw_i, float2* tw_a, cudaStream_t s);
+cudaError_t launch_small_tw(int lgN, float2* tw, cudaStream_t s);   // small_tw_count(lgN) values
+// Pair-operator tables of one instance from its FP64 spectrum: tA, tB n/4 + 1
+// values, tc, abs2 n/2 + 1 (null: no ADMM).
+cudaError_t launch_small_tables(const double2* chat, int64_t n, float4* tA, float2* tB, float2* tc, double* abs2,
+                                cudaStream_t s);
+
+// Size classes of a batch: one CTA per instance (ISTA lgN = lgn - 1, ADMM
+// lgN = lgn; n <= 8192 for both).
+struct SmallInst {
+  const float4* tA;
+  const float2 *tB, *tc;
+  const float* tb;
+  const float2 *tw_i, *tw_a, *tw;
+  const int32_t* rows;
+  int* status;
+  int64_t noff, moff;      // x / z and y in the caller's concatenated vectors
+  int m, id;               // id: the instance's scalars
+};
+struct SmallScalars {      // per call and instance
+  float thr, tau, rho, sigma, tau1, tau2, d_on, d_off;
+};
+cudaError_t launch_small_class(bool admm, int lgN, const SmallInst* inst, int count, const SmallScalars* sc,
+                               const float* y, float* xz, int iters, cudaStream_t s);
 
 // One plan of a grouped (batched) solve: what the grouped element-wise
 // kernels need of it.

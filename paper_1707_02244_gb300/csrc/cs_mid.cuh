@@ -144,12 +144,16 @@ __device__ __forceinline__ void op_admm(const float2 ch, const float bb, float r
 // packed and the complex geometry of a 4096 x 4096 image.
 // SHAPE 10 + LGN1 (1D) and 30 + LGN1 (2D), LGN1 = 6 .. 10: radix-8 tiles of
 // one row pair (two for LGN1 = 6), 8 values per thread.
+// SHAPE 50 + LGN1 (1D, LGN1 = 7 .. 9): 4096-value tiles, 16 values per thread
+// (grouped launches).
 template <int SHAPE> struct MidShape {
-  static_assert((SHAPE >= 16 && SHAPE <= 20) || (SHAPE >= 36 && SHAPE <= 40), "radix-8 mid shapes");
-  static constexpr bool kTwoD = SHAPE >= 30;
-  static constexpr int kLgN1 = SHAPE - (kTwoD ? 30 : 10), kLgU = kLgN1 == 6 ? 1 : 0;
-  static constexpr int kLgR = 3, kVpt = VPT8;
-  using Lay = StaticLayout<kLgN1, kLgU + 1, false, 3>;
+  static_assert((SHAPE >= 16 && SHAPE <= 20) || (SHAPE >= 36 && SHAPE <= 40) || (SHAPE >= 57 && SHAPE <= 59),
+                "mid shapes");
+  static constexpr bool kTwoD = SHAPE >= 30 && SHAPE <= 40, kR8 = SHAPE < 50;
+  static constexpr int kLgN1 = SHAPE - (kTwoD ? 30 : kR8 ? 10 : 50);
+  static constexpr int kLgU = kR8 ? (kLgN1 == 6 ? 1 : 0) : 11 - kLgN1;
+  static constexpr int kLgR = kR8 ? 3 : 4, kVpt = kR8 ? VPT8 : EPT;
+  using Lay = StaticLayout<kLgN1, kLgU + 1, false, kLgR>;
   __device__ static Lay lay(const Geo&) { return Lay{}; }
   __device__ static constexpr int lgN1(const Geo&) { return kLgN1; }
   __device__ static constexpr int lgU(const Geo&) { return kLgU; }

@@ -17,7 +17,9 @@ namespace {
 __device__ __forceinline__ float soft(float u, float g) { return u > g ? u - g : (u < -g ? u + g : 0.f); }
 
 // Product operator on a pair of the packed spectrum (a, a', b in tA, tB; see
-// the single-vector table kernel): C^T for ADJ, else C.
+// the table kernel below): C^T for ADJ, else C.
+//   C^T: Z_k' = a Z_k + b conj(Z_{N-k}), Z_{N-k}' = a' Z_{N-k} - conj(b) conj(Z_k)
+//   C:   a, a' conjugated and b -> -conj(b)
 template <bool ADJ>
 struct OpReal {
   const float4* tA;
@@ -25,8 +27,6 @@ struct OpReal {
   __device__ __forceinline__ void operator()(int k, float2& za, float2& zb) const {
     const float4 t = __ldg(tA + k);
     const float2 be = __ldg(tB + k);
-    // C^T: Z_k' = a Z_k + b conj(Z_{N-k}), Z_{N-k}' = a' Z_{N-k} - conj(b) conj(Z_k);
-    // C: a, a' conjugated and b -> -conj(b)
     const float2 al = make_float2(t.x, ADJ ? t.y : -t.y), al2 = make_float2(t.z, ADJ ? t.w : -t.w);
     const float2 b1 = ADJ ? be : make_float2(-be.x, be.y);
     const float2 b2 = make_float2(-b1.x, b1.y);
@@ -90,10 +90,10 @@ __device__ __forceinline__ void stage_y(const SmallArgs& a, int n, float* yd, ui
   __syncthreads();
 }
 
-// ISTA (Algorithm 1): n = 2 N packed, x (natural order, 8-byte aligned) in
-// and out.
+// ISTA (Algorithm 1): n = 2 N packed, x (natural order, any 4-byte boundary)
+// in and out.
 template <int LG>
-__global__ void __launch_bounds__(SmallShape<LG>::NT) small_ista_k(const SmallArgs a) {
+__device__ __forceinline__ void small_ista(const SmallArgs& a) {
   using S = SmallShape<LG>;
   constexpr int N = S::N, E = S::E, ST = N / E, NT = S::NT;
   extern __shared__ float2 sm[];
@@ -105,23 +105,24 @@ __global__ void __launch_bounds__(SmallShape<LG>::NT) small_ista_k(const SmallAr
   stage_y<NT>(a, 2 * N, reinterpret_cast<float*>(yd), mk);
   const int tid = threadIdx.x;
   const bool act = tid < S::NA;
-  float2* xg = reinterpret_cast<float2*>(a.x);
   float2 x[E], v[E];
   uint32_t mb = 0;
   if (act) {
 #pragma unroll
     for (int r = 0; r < E; ++r) {
       const int p = tid + r * ST;
-      x[r] = v[r] = xg[p];
+      x[r] = v[r] = make_float2(a.x[2 * p], a.x[2 * p + 1]);
       mb |= ((mk[p >> 4] >> ((2 * p) & 31)) & 3u) << (2 * r);
     }
   }
   const OpReal<false> opf{a.tA, a.tB};
   const OpReal<true> opa{a.tA, a.tB};
+  // (one copy of the transform with the product's sign as a run-time factor
+  // was slower, 4.7 against 4.0 us an iteration at n = 4096)
 #pragma unroll 1
   for (int it = 0; it < a.iters; ++it) {
     const bool st = a.stats != nullptr && it + 1 == a.iters;
-    float r2 = 0.f, dx2 = 0.f, x2 = 0.f, l1 = 0.f, er = 0.f, nf = 0.f;
+    float r2 = 0.f;
     small_conv<LG>(v, S0, S1, tw, opf);
     if (act) {
 #pragma unroll
@@ -134,6 +135,7 @@ __global__ void __launch_bounds__(SmallShape<LG>::NT) small_ista_k(const SmallAr
       }
     }
     small_conv<LG>(v, S0, S1, tw, opa);
+    float dx2 = 0.f, x2 = 0.f, l1 = 0.f, er = 0.f, nf = 0.f;
     if (act) {
 #pragma unroll
       for (int r = 0; r < E; ++r) {
@@ -167,19 +169,23 @@ __global__ void __launch_bounds__(SmallShape<LG>::NT) small_ista_k(const SmallAr
   }
   if (act) {
 #pragma unroll
-    for (int r = 0; r < E; ++r) xg[tid + r * ST] = x[r];
+    for (int r = 0; r < E; ++r) {
+      const int p = tid + r * ST;
+      a.x[2 * p] = x[r].x;
+      a.x[2 * p + 1] = x[r].y;
+    }
   }
 }
 
 // Algorithm 3, n = N (complex): state (v, z, mu, nu) in natural order, in
 // when a.warm (else zero), out where the pointer is not null.
 template <int LG>
-__global__ void __launch_bounds__(SmallShape<LG>::NT) small_admm_k(const SmallArgs a) {
+__device__ __forceinline__ void small_admm(const SmallArgs& a) {
   using S = SmallShape<LG>;
   constexpr int N = S::N, E = S::E, ST = N / E, NT = S::NT;
   extern __shared__ float2 sm[];
   float2 *S0 = sm, *S1 = S0 + small_buf<LG>(), *tw = S1 + small_buf<LG>();
-  float* yd = reinterpret_cast<float*>(tw + ((S::kTw + 1) & ~1));
+  float* yd = reinterpret_cast<float*>(S1);   // only until the registers hold it
   __shared__ uint32_t mk[N / 32];
   __shared__ double red[NT / 32];
   load_tw<LG>(tw, a.tw);
@@ -250,6 +256,56 @@ __global__ void __launch_bounds__(SmallShape<LG>::NT) small_admm_k(const SmallAr
       }
     }
   }
+}
+
+template <int LG>
+__global__ void __launch_bounds__(SmallShape<LG>::NT) small_ista_k(const SmallArgs a) { small_ista<LG>(a); }
+template <int LG>
+__global__ void __launch_bounds__(SmallShape<LG>::NT) small_admm_k(const SmallArgs a) { small_admm<LG>(a); }
+
+// Instance blockIdx.x of a size class of a batch: its constants, its scalars
+// of this call, and the call's concatenated vectors.
+__device__ __forceinline__ SmallArgs class_args(const SmallInst& d, const SmallScalars& s, const float* y, int iters) {
+  SmallArgs a{};
+  a.tA = d.tA;
+  a.tB = d.tB;
+  a.tc = d.tc;
+  a.tb = d.tb;
+  a.tw = d.tw;
+  a.rows = d.rows;
+  a.m = d.m;
+  a.y = y + d.moff;
+  a.status = d.status;
+  a.iters = iters;
+  a.thr = s.thr;
+  a.tau = s.tau;
+  a.rho = s.rho;
+  a.sigma = s.sigma;
+  a.tau1 = s.tau1;
+  a.tau2 = s.tau2;
+  a.d_on = s.d_on;
+  a.d_off = s.d_off;
+  return a;
+}
+template <int LG>
+__global__ void __launch_bounds__(SmallShape<LG>::NT)
+    class_ista_k(const SmallInst* __restrict__ inst, const SmallScalars* __restrict__ sc, const float* __restrict__ y,
+                 float* __restrict__ x, int iters) {
+  SmallInst d = inst[blockIdx.x];
+  d.tw = d.tw_i;
+  SmallArgs a = class_args(d, sc[d.id], y, iters);
+  a.x = x + d.noff;
+  small_ista<LG>(a);
+}
+template <int LG>
+__global__ void __launch_bounds__(SmallShape<LG>::NT)
+    class_admm_k(const SmallInst* __restrict__ inst, const SmallScalars* __restrict__ sc, const float* __restrict__ y,
+                 float* __restrict__ z, int iters) {
+  SmallInst d = inst[blockIdx.x];
+  d.tw = d.tw_a;
+  SmallArgs a = class_args(d, sc[d.id], y, iters);
+  a.z = z + d.noff;
+  small_admm<LG>(a);
 }
 
 // Power iteration on A^T A from the fixed start vector in a.x (natural
@@ -403,9 +459,30 @@ __global__ void small_tab_admm_k(const double2* __restrict__ chat, int64_t n, fl
 }
 
 template <int LG>
-constexpr size_t small_smem(bool dense, bool admm) {
+constexpr size_t small_smem(bool dense) {
   return sizeof(float2) * (2 * small_buf<LG>() + ((SmallShape<LG>::kTw + 1) & ~1)) +
-         (dense ? sizeof(float) * (size_t)(admm ? 1 : 2) * (1 << LG) : 0);
+         (dense ? sizeof(float2) << LG : 0);
+}
+
+cudaError_t opt_in_smem(const void* fn, size_t smem) {
+  return smem > 48 * 1024 ? cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                          : cudaSuccess;
+}
+
+// LG = 13 (64 values of padding per 1024 and 62 KiB of twiddles: 201 KiB)
+// fits without a dense y, so only ADMM takes it.
+template <int LG>
+cudaError_t class_run(bool admm, const SmallInst* inst, int count, const SmallScalars* sc, const float* y, float* xz,
+                      int iters, cudaStream_t s) {
+  const void* fn = nullptr;
+  size_t smem = small_smem<LG>(!admm);
+  if (admm) fn = (const void*)class_admm_k<LG>;
+  else if constexpr (LG <= SMALL_LG_MAX) fn = (const void*)class_ista_k<LG>;
+  if (!fn) return cudaErrorInvalidValue;
+  const cudaError_t e = opt_in_smem(fn, smem);
+  if (e != cudaSuccess) return e;
+  void* args[] = {&inst, &sc, &y, &xz, &iters};
+  return cudaLaunchKernel(fn, dim3((unsigned)count), dim3(SmallShape<LG>::NT), args, smem, s);
 }
 
 template <int LG>
@@ -414,16 +491,14 @@ cudaError_t small_run(SmallKind kind, const SmallArgs& a, cudaStream_t s) {
   const void* fn = nullptr;
   size_t smem = 0;
   switch (kind) {
-    case SMALL_ISTA: fn = (const void*)small_ista_k<LG>; smem = small_smem<LG>(true, false); break;
-    case SMALL_ADMM: fn = (const void*)small_admm_k<LG>; smem = small_smem<LG>(true, true); break;
-    case SMALL_POWER: fn = (const void*)small_power_k<LG>; smem = small_smem<LG>(false, false); break;
-    case SMALL_FWD: fn = (const void*)small_product_k<LG, true>; smem = small_smem<LG>(true, false); break;
-    case SMALL_ADJ: fn = (const void*)small_product_k<LG, false>; smem = small_smem<LG>(true, false); break;
+    case SMALL_ISTA: fn = (const void*)small_ista_k<LG>; smem = small_smem<LG>(true); break;
+    case SMALL_ADMM: fn = (const void*)small_admm_k<LG>; smem = small_smem<LG>(false); break;
+    case SMALL_POWER: fn = (const void*)small_power_k<LG>; smem = small_smem<LG>(false); break;
+    case SMALL_FWD: fn = (const void*)small_product_k<LG, true>; smem = small_smem<LG>(true); break;
+    case SMALL_ADJ: fn = (const void*)small_product_k<LG, false>; smem = small_smem<LG>(true); break;
   }
-  if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = opt_in_smem(fn, smem);
+  if (e != cudaSuccess) return e;
   void* args[] = {const_cast<SmallArgs*>(&a)};
   return cudaLaunchKernel(fn, dim3(1), dim3(S::NT), args, smem, s);
 }
@@ -441,8 +516,20 @@ cudaError_t launch_small(SmallKind kind, int lgN, const SmallArgs& a, cudaStream
   return cudaErrorInvalidValue;
 }
 
+cudaError_t launch_small_class(bool admm, int lgN, const SmallInst* inst, int count, const SmallScalars* sc,
+                               const float* y, float* xz, int iters, cudaStream_t s) {
+  switch (lgN) {
+#define CS_X(L) case L: return class_run<L>(admm, inst, count, sc, y, xz, iters, s);
+    CS_SMALL_LG(CS_X)
+    CS_X(13)
+#undef CS_X
+  }
+  return cudaErrorInvalidValue;
+}
+
 static SmallTwStages tw_stages(int lgN) {
   switch (lgN) {
+    case 13: return small_tw_stages<13>();
 #define CS_X(L) case L: return small_tw_stages<L>();
     CS_SMALL_LG(CS_X)
 #undef CS_X
@@ -452,17 +539,17 @@ static SmallTwStages tw_stages(int lgN) {
 
 int small_tw_count(int lgN) { return tw_stages(lgN).total; }
 
-cudaError_t launch_small_tables(const double2* chat, int64_t n, int lgn, float4* tA, float2* tB, float2* tc,
-                                double* abs2, float2* tw_i, float2* tw_a, cudaStream_t s) {
+cudaError_t launch_small_tw(int lgN, float2* tw, cudaStream_t s) {
+  const SmallTwStages d = tw_stages(lgN);
+  small_tw_k<<<(unsigned)((d.total + 255) / 256), 256, 0, s>>>(tw, d);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_small_tables(const double2* chat, int64_t n, float4* tA, float2* tB, float2* tc, double* abs2,
+                                cudaStream_t s) {
   auto nb = [](int64_t c) { return (unsigned)((c + 255) / 256); };
   small_tab_ista_k<<<nb(n / 4 + 1), 256, 0, s>>>(chat, n, tA, tB);
-  const SmallTwStages di = tw_stages(lgn - 1);
-  small_tw_k<<<nb(di.total), 256, 0, s>>>(tw_i, di);
-  if (tc) {
-    small_tab_admm_k<<<nb(n / 2 + 1), 256, 0, s>>>(chat, n, tc, abs2);
-    const SmallTwStages da = tw_stages(lgn);
-    small_tw_k<<<nb(da.total), 256, 0, s>>>(tw_a, da);
-  }
+  if (tc) small_tab_admm_k<<<nb(n / 2 + 1), 256, 0, s>>>(chat, n, tc, abs2);
   return cudaGetLastError();
 }
 
