@@ -14,7 +14,7 @@ SRC = PKG / "csrc"
 OBJ = PKG / "_build"
 LIB = PKG / "libcsgb.so"
 SOURCES = ["cs_col.cu", "cs_col8a.cu", "cs_col8b.cu", "cs_mid.cu", "cs_mid8.cu", "cs_aux.cu", "cs_api.cu", "cs_static.cu",
-           "cs_batch.cu", "cs_group.cu", "cs_small.cu", "cs_smooth.cu", "cs_direct.cu"]
+           "cs_batch.cu", "cs_cluster.cu", "cs_group.cu", "cs_small.cu", "cs_smooth.cu", "cs_direct.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2", "-I", str(ROOT / "include")]
 

@@ -70,6 +70,7 @@ struct cs_plan_s {
     double* abs2 = nullptr;
     float* tb = nullptr;
   } sml;
+  bool cluster_i = false, cluster_a = false;   // one cluster solves the instance
   CallArgs last_ca{};              // arguments of the last single-CTA solve: cs_profile_pass sends them first
   bool ca_stale = false;
   // unrolled-ISTA gradient (cs_grad): allocated at the first call, grown on demand
@@ -452,6 +453,21 @@ SmallArgs small_args(const cs_plan_s* p, bool admm) {
   return a;
 }
 
+ClusterArgs cluster_args(const cs_plan_s* p, bool admm) {
+  ClusterArgs a{};
+  a.geo = admm ? p->ga : p->gi;
+  const cs_plan_s::Sel& sel = admm ? p->sa : p->si;
+  a.mask = sel.mask;
+  a.prefix = sel.prefix;
+  a.ys = sel.ys;
+  a.tab_i = p->tab_ista;
+  a.tab_c = p->tab_admm_c;
+  a.tab_b = p->tab_admm_b;
+  a.xtrue = p->xtrue ? (admm ? p->xt_a : p->xt_i) : nullptr;
+  a.partials = p->partials;
+  return a;
+}
+
 // B's spectrum 1 / (n (rho |c^|^2 + sigma)) of the plan, tabulated when it
 // holds another pair.
 cudaError_t admm_table(cs_plan_s* p, double rho, double sigma, cudaStream_t s, int* launches) {
@@ -639,6 +655,8 @@ cs_status build_plan(cs_plan_t* out, int64_t n0, int64_t n1, int64_t m, const in
     CS_PLAN_TRY(launch_small_tw(lgn - 1, p->sml.tw_i, s));
     if (p->small_a) CS_PLAN_TRY(launch_small_tw(lgn, p->sml.tw_a, s));
   }
+  p->cluster_i = !p->small_i && small_tiles && cluster_init(p->gi, false);
+  p->cluster_a = !p->small_a && small_tiles && cluster_init(p->ga, true);
   CS_PLAN_TRY(admm_table(p, 1.0, 1.0, s, nullptr));
   CS_PLAN_TRY(launch_build_mask(d_rows, m, n, p->gi, 1, p->si.mask, p->status, s));
   CS_PLAN_TRY(launch_build_mask(d_rows, m, n, p->ga, 0, p->sa.mask, p->status, s));
@@ -693,6 +711,14 @@ cs_status cs_forward(cs_plan_t p, const float* x, float* y) {
     CS_TRY(launch_small(SMALL_FWD, p->lgn - 1, sa, s));
     return CS_OK;
   }
+  if (p->cluster_i) {
+    ClusterArgs ca = cluster_args(p, false);
+    ca.x = const_cast<float*>(x);
+    ca.z = p->dense;
+    CS_TRY(launch_cluster(CLUSTER_FWD, ca, s));
+    CS_TRY(launch_gather_rows(p->dense, p->rows32, p->m, y, s));
+    return CS_OK;
+  }
   CallArgs a{};
   a.src = x;
   a.dst = p->dense;
@@ -717,6 +743,14 @@ cs_status cs_adjoint(cs_plan_t p, const float* r, float* x) {
   }
   CS_TRY(cudaMemsetAsync(p->dense, 0, p->n * sizeof(float), s));
   CS_TRY(launch_scatter_rows(r, p->rows32, p->m, p->dense, s));
+  if (p->cluster_i) {
+    p->ista_args = p->admm_args = false;
+    ClusterArgs ca = cluster_args(p, false);
+    ca.x = p->dense;
+    ca.z = x;
+    CS_TRY(launch_cluster(CLUSTER_ADJ, ca, s));
+    return CS_OK;
+  }
   CallArgs a{};
   a.src = p->dense;
   a.dst = x;
@@ -739,6 +773,17 @@ cs_status cs_opnorm2(cs_plan_t p, int iters, double* L) {
     sa.stats = p->stats;
     sa.iters = iters;
     CS_TRY(launch_small(SMALL_POWER, p->lgn - 1, sa, s));
+    CS_TRY(read_back(p));
+    *L = p->host_stats[ST_DX2];
+    return latched_status(p);
+  }
+  if (p->cluster_i) {
+    p->ista_args = p->admm_args = false;
+    ClusterArgs ca = cluster_args(p, false);
+    ca.x = p->dense2;
+    ca.stats = p->stats;
+    ca.iters = iters;
+    CS_TRY(launch_cluster(CLUSTER_POWER, ca, s));
     CS_TRY(read_back(p));
     *L = p->host_stats[ST_DX2];
     return latched_status(p);
@@ -815,13 +860,30 @@ cs_status cs_ista(cs_plan_t p, const float* y, float lambda, float tau, int iter
                         p->launches += 1;
                         return launch_small(SMALL_ISTA, p->lgn - 1, sa, s);
                       }));
+  } else if (p->cluster_i && iters > 0) {
+    CS_TRY(launch_scatter_y(y, p->si.pos, p->m, p->si.ys, p->status, s));
+    p->launches += 1;
+    ClusterArgs ca = cluster_args(p, false);
+    ca.x = x;
+    ca.thr = a.thr;
+    ca.tau = tau;
+    p->last_ca = a;
+    p->ca_stale = true;
+    CS_TRY(solve_loop(p, iters, &run, &conv, stats != nullptr, SMALL_CHUNK,
+                      [&](int, int len, bool, bool st) {
+                        ca.iters = len;
+                        ca.stats = st ? p->stats : nullptr;
+                        p->launches += st ? 2 : 1;
+                        const cudaError_t e = launch_cluster(CLUSTER_ISTA, ca, s);
+                        return e == cudaSuccess && st ? launch_finalize(p->partials, cluster_ctas(), p->stats, s) : e;
+                      }));
   } else {
     p->ca_stale = false;
     CS_TRY(launch_set_args(a, p->ca, s));
     CS_TRY(launch_scatter_y(y, p->si.pos, p->m, p->si.ys, p->status, s));
     p->launches += 2;
   }
-  if (!p->small_i && iters > 0) {
+  if (!p->small_i && !p->cluster_i && iters > 0) {
     CS_TRY(launch_to_tile(x, p->xi_t, p->gi, 1, s));
     CS_TRY(launch_col(COL_LOAD, kparams(p, p->gi, 0), s));
     p->launches += 2;
@@ -861,7 +923,7 @@ cs_status admm_impl(cs_plan_t p, const float* y, float lambda, const cs_admm_par
   p->launches = 0;
   float* tiled[4] = {p->av, p->az, p->amu, p->anu};
   float* natural[4] = {v, z, mu, nu};
-  const bool small = p->small_a && iters > 0;
+  const bool small = (p->small_a || p->cluster_a) && iters > 0;   // one launch, state in natural order
   for (int i = 0; i < 4 && !small; ++i) {
     if (warm) {
       CS_TRY(launch_to_tile(natural[i], tiled[i], p->ga, 0, s));
@@ -891,30 +953,52 @@ cs_status admm_impl(cs_plan_t p, const float* y, float lambda, const cs_admm_par
   if (small) {
     p->last_ca = a;
     p->ca_stale = true;
-    SmallArgs sa = small_args(p, true);
-    sa.y = y;
-    sa.thr = a.thr;
-    sa.rho = a.rho;
-    sa.sigma = a.sigma;
-    sa.tau1 = a.tau1;
-    sa.tau2 = a.tau2;
-    sa.d_on = a.d_on;
-    sa.d_off = a.d_off;
+    SmallArgs sa{};
+    ClusterArgs ca{};
+    auto fill = [&](auto& q) {
+      q.thr = a.thr;
+      q.rho = a.rho;
+      q.sigma = a.sigma;
+      q.tau1 = a.tau1;
+      q.tau2 = a.tau2;
+      q.d_on = a.d_on;
+      q.d_off = a.d_off;
+    };
+    if (p->small_a) {
+      sa = small_args(p, true);
+      sa.y = y;
+      fill(sa);
+    } else {
+      CS_TRY(launch_scatter_y(y, p->sa.pos, p->m, p->sa.ys, p->status, s));
+      p->launches += 1;
+      ca = cluster_args(p, true);
+      fill(ca);
+    }
     // a chunk that another one may follow leaves its state in the caller's
     // vectors, or in the plan's where the caller takes none
     const bool watch = p->xtrue != nullptr && p->tol > 0.0;
     CS_TRY(solve_loop(p, iters, &run, &conv, stats != nullptr, SMALL_CHUNK, [&](int done, int len, bool fin, bool st) {
       const bool carry = watch || !fin || done > 0;
-      sa.v = v ? v : carry ? p->av : nullptr;
-      sa.z = z ? z : carry ? p->az : nullptr;
-      sa.mu = mu ? mu : carry ? p->amu : nullptr;
-      sa.nu = nu ? nu : carry ? p->anu : nullptr;
-      sa.x = x;
-      sa.warm = warm || done > 0;
-      sa.iters = len;
-      sa.stats = st ? p->stats : nullptr;
+      auto step = [&](auto& q) {
+        q.v = v ? v : carry ? p->av : nullptr;
+        q.z = z ? z : carry ? p->az : nullptr;
+        q.mu = mu ? mu : carry ? p->amu : nullptr;
+        q.nu = nu ? nu : carry ? p->anu : nullptr;
+        q.x = x;
+        q.warm = warm || done > 0;
+        q.iters = len;
+        q.stats = st ? p->stats : nullptr;
+      };
       p->launches += 1;
-      return launch_small(SMALL_ADMM, p->lgn, sa, s);
+      if (p->small_a) {
+        step(sa);
+        return launch_small(SMALL_ADMM, p->lgn, sa, s);
+      }
+      step(ca);
+      const cudaError_t e = launch_cluster(CLUSTER_ADMM, ca, s);
+      if (e != cudaSuccess || !st) return e;
+      p->launches += 1;
+      return launch_finalize(p->partials, cluster_ctas(), p->stats, s);
     }));
   } else {
     p->ca_stale = false;

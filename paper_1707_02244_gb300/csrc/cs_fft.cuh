@@ -131,6 +131,7 @@ struct DynLayout {
   __device__ __forceinline__ int LG() const { return lgL; }
   __device__ __forceinline__ int NV() const { return lgnv; }
   __device__ __forceinline__ bool VF() const { return vec_fast; }
+  __device__ __forceinline__ int tid() const { return threadIdx.x; }
   __device__ __forceinline__ int at(int vec, int idx) const {
     return vec_fast ? ((idx << lgnv) + vec) : ((vec << lgL) + idx);
   }
@@ -144,6 +145,7 @@ struct StaticLayout {
   __device__ __forceinline__ constexpr int LG() const { return LGL; }
   __device__ __forceinline__ constexpr int NV() const { return LGNV; }
   __device__ __forceinline__ constexpr bool VF() const { return VEC_FAST; }
+  __device__ __forceinline__ int tid() const { return threadIdx.x; }
   __device__ __forceinline__ int at(int vec, int idx) const {
     return VEC_FAST ? ((idx << LGNV) + vec) : ((vec << LGL) + idx);
   }
@@ -160,6 +162,16 @@ struct StaticLayout {
   __device__ __forceinline__ static constexpr int padV(int vec) {
     return VEC_FAST ? vec + (vec >> 4) : vec * ((1 << LGL) + (1 << (LGL - 4)));
   }
+};
+
+// The same for a kernel that loops over whole transforms: the thread index is
+// threadIdx.x + zero with a zero the compiler cannot know (read from shared
+// memory), so that the addresses of every stage are recomputed instead of
+// kept in registers across the loop, where they would spill.
+template <class L> struct LoopLayout : L {
+  int zero;
+  __device__ __forceinline__ explicit LoopLayout(int z) : zero(z) {}
+  __device__ __forceinline__ int tid() const { return threadIdx.x + zero; }
 };
 
 // Element hooks: `pre` runs on the values a first stage loads (before its
@@ -269,11 +281,12 @@ __device__ __forceinline__ void stockham_stage(float2* s, const LAY& lay, int lg
   const int lgstep = lgLt - lgLs - lgR;          // w_{Ls R}^(r k) = tw[(r k) << lgstep]
   const bool first = lgLs == 0;
   const bool last = lgLs + lgR == lgL;
+  const int tid = lay.tid();
   float2 v[BPT][R];
   int vecs[BPT], js[BPT];
 #pragma unroll
   for (int i = 0; i < BPT; ++i) {
-    const int b = threadIdx.x + i * NT;
+    const int b = tid + i * NT;
     if (lay.VF()) { vecs[i] = b & ((1 << lgnv) - 1); js[i] = b >> lgnv; }
     else { vecs[i] = b >> lgLR; js[i] = b & ((1 << lgLR) - 1); }
     if (b < nb) {
@@ -293,7 +306,7 @@ __device__ __forceinline__ void stockham_stage(float2* s, const LAY& lay, int lg
   if constexpr (!IN::kGlobal) __syncthreads();
 #pragma unroll
   for (int i = 0; i < BPT; ++i) {
-    const int b = threadIdx.x + i * NT;
+    const int b = tid + i * NT;
     if (b < nb) {
       const int j = js[i];
       const int k = j & (Ls - 1);

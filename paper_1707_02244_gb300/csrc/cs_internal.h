@@ -240,6 +240,27 @@ struct SmallScalars {      // per call and instance
 cudaError_t launch_small_class(bool admm, int lgN, const SmallInst* inst, int count, const SmallScalars* sc,
                                const float* y, float* xz, int iters, cudaStream_t s);
 
+// Solves and products of middle-sized instances by one cluster of CTAs
+// (cs_cluster.cu); geo the radix-8 geometry (packed, or complex-n for ADMM).
+enum ClusterKind : int { CLUSTER_ISTA, CLUSTER_ADMM, CLUSTER_POWER, CLUSTER_FWD, CLUSTER_ADJ };
+struct ClusterArgs {
+  Geo geo;
+  const uint32_t *mask, *prefix;   // rows of Omega and compact y in the plan's tile order
+  const float* ys;
+  const float4* tab_i;
+  const float2* tab_c;
+  const float* tab_b;
+  float *x, *z, *mu, *nu, *v;      // natural order (ISTA: x; ADMM: the state, null not returned; products: x -> z)
+  const float* xtrue;              // tile order, or null
+  double* partials;                // per CTA, with stats
+  double* stats;                   // null: no statistics (power iteration: the sums themselves)
+  int iters, warm;
+  float thr, tau, rho, sigma, tau1, tau2, d_on, d_off;
+};
+bool cluster_init(const Geo& g, bool admm);
+cudaError_t launch_cluster(ClusterKind kind, const ClusterArgs& a, cudaStream_t s);
+int cluster_ctas();
+
 // One plan of a grouped (batched) solve: what the grouped element-wise
 // kernels need of it.
 struct GroupDesc {
