@@ -78,10 +78,10 @@ struct cs_plan_s {
     int ck_cap = 0, seg_cap = 0;
     float* ckpt = nullptr;   // [ck_cap][n]  x(sK), tile order
     float* seg = nullptr;    // [seg_cap + 1][n]  x(t) of the segment being replayed
-    float* rseg = nullptr;   // [seg_cap][n]  r(t) of the segment
-    float *g = nullptr, *w = nullptr, *q = nullptr;
+    float2* rw = nullptr;    // [seg_cap][n/2]  column transform of r(t)
+    float2* xw = nullptr;    // [seg_cap][n/2]  column transform of x(t)
+    float *g = nullptr, *w = nullptr;
     float* dy = nullptr;     // [m] dL/dy, compact in the tile order of the rows
-    float2* W2 = nullptr;
     float4* gacc = nullptr;  // spectrum of dL/dc (before tau), per pair slot
     double* gpart = nullptr; // per column CTA: dL/dtheta
     CallArgs* ca = nullptr;  // [seg_cap + 1]: step j of a segment, and the output pass
@@ -235,7 +235,7 @@ void free_plan(cs_plan_s* p) {
   void* sbufs[] = {p->sml.tA, p->sml.tB, p->sml.tc, p->sml.tw_i, p->sml.tw_a, p->sml.abs2, p->sml.tb};
   for (void* b : sbufs)
     if (b) cudaFree(b);
-  void* gbufs[] = {p->gr.ckpt, p->gr.seg, p->gr.rseg, p->gr.g, p->gr.w, p->gr.q, p->gr.dy, p->gr.W2, p->gr.gacc,
+  void* gbufs[] = {p->gr.ckpt, p->gr.seg, p->gr.rw, p->gr.xw, p->gr.g, p->gr.w, p->gr.dy, p->gr.gacc,
                    p->gr.gpart, p->gr.ca};
   for (void* b : gbufs)
     if (b) cudaFree(b);
@@ -255,6 +255,7 @@ KParams kparams(const cs_plan_s* p, const Geo& g, int flags) {
   KParams k;
   k.geo = g;
   k.pp.W = p->W;
+  k.pp.Wi = p->W;
   const cs_plan_s::Sel& sel = (&g == &p->gi) ? p->si : p->sa;
   k.pp.mask = sel.mask;
   k.pp.prefix = sel.prefix;
@@ -265,7 +266,7 @@ KParams kparams(const cs_plan_s* p, const Geo& g, int flags) {
   k.pp.tab_admm_c = p->tab_admm_c;
   k.pp.tab_admm_b = p->tab_admm_b;
   k.pp.status = p->status;
-  k.pp.W2 = p->gr.W2;
+  k.pp.W2 = nullptr;
   k.pp.gacc = p->gr.gacc;
   k.pp.gpart = p->gr.gpart;
   k.ca = p->ca;
@@ -1102,19 +1103,18 @@ cudaError_t grad_reserve(cs_plan_s* p, int ck, int seg) {
     }
   }
   const int nck = ck > G.ck_cap ? ck : G.ck_cap, nseg = seg > G.seg_cap ? seg : G.seg_cap;
-  void* old[] = {G.ckpt, G.seg, G.rseg, G.g, G.w, G.q, G.dy, G.W2, G.gacc, G.gpart, G.ca};
+  void* old[] = {G.ckpt, G.seg, G.rw, G.xw, G.g, G.w, G.dy, G.gacc, G.gpart, G.ca};
   for (void* b : old)
     if (b) cudaFree(b);
   G = cs_plan_s::Grad{};
   const size_t n = (size_t)p->n;
   e = dalloc(&G.ckpt, (size_t)nck * n);
   if (e == cudaSuccess) e = dalloc(&G.seg, (size_t)(nseg + 1) * n);
-  if (e == cudaSuccess) e = dalloc(&G.rseg, (size_t)nseg * n);
+  if (e == cudaSuccess) e = dalloc(&G.rw, (size_t)nseg * (n / 2));
+  if (e == cudaSuccess) e = dalloc(&G.xw, (size_t)nseg * (n / 2));
   if (e == cudaSuccess) e = dalloc(&G.g, n);
   if (e == cudaSuccess) e = dalloc(&G.w, n);
-  if (e == cudaSuccess) e = dalloc(&G.q, n);
   if (e == cudaSuccess) e = dalloc(&G.dy, (size_t)p->m);
-  if (e == cudaSuccess) e = dalloc(&G.W2, n / 2);
   if (e == cudaSuccess) e = dalloc(&G.gacc, (size_t)tab_count(p->gi));
   if (e == cudaSuccess) e = dalloc(&G.gpart, (size_t)p->gi.col_ctas);
   if (e == cudaSuccess) e = dalloc(&G.ca, (size_t)nseg + 1);
@@ -1149,42 +1149,47 @@ cudaError_t run_graph(cs_plan_s* p, uint64_t key, F&& enqueue) {
   return cudaGraphLaunch(it->second, p->stream);
 }
 
-KParams kp_step(const cs_plan_s* p, int j, int flags) {
-  KParams k = kparams(p, p->gi, flags);
+// Pass parameters of step j: from exchange buffer `in` to `out` (null: W),
+// correlated with the transform in w2.
+KParams kp_step(const cs_plan_s* p, int j, const float2* in = nullptr, float2* out = nullptr,
+                const float2* w2 = nullptr) {
+  KParams k = kparams(p, p->gi, 0);
   k.ca = p->gr.ca + j;
+  if (in) k.pp.Wi = in;
+  if (out) k.pp.W = out;
+  k.pp.W2 = w2;
   return k;
 }
 
-// Replay of one segment: x(0) of the segment in seg[0]; step j writes r(j)
-// and x(j+1).
+// Replay of one segment of L steps: x(0) of the segment in seg[0]; step j
+// writes x(j+1) and leaves the column transforms of x(j) and r(j) in xw and
+// rw (the passes that follow read them there).
 cudaError_t enqueue_replay(cs_plan_s* p, int L, cudaStream_t s) {
-  const Geo& g = p->gi;
-  cudaError_t e = launch_col(COL_LOADT, kp_step(p, 0, 0), s);
+  auto& G = p->gr;
+  const size_t h = (size_t)p->n / 2;
+  cudaError_t e = launch_col(COL_LOADT, kp_step(p, 0, nullptr, G.xw), s);
   for (int j = 0; j < L && e == cudaSuccess; ++j) {
-    e = launch_mid(MID_FWD, kp_step(p, j, 0), s);
-    if (e == cudaSuccess) e = launch_col(COL_RES_SAVE, kp_step(p, j, 0), s);
-    if (e == cudaSuccess) e = launch_mid(MID_ADJ, kp_step(p, j, 0), s);
-    if (e == cudaSuccess) e = launch_col(COL_ISTA_SEG, kp_step(p, j, 0), s);
+    e = launch_mid(MID_FWD, kp_step(p, j, G.xw + j * h), s);
+    if (e == cudaSuccess) e = launch_col(COL_RESIDUAL, kp_step(p, j, nullptr, G.rw + j * h), s);
+    if (e == cudaSuccess) e = launch_mid(MID_ADJ, kp_step(p, j, G.rw + j * h), s);
+    if (e == cudaSuccess)
+      e = launch_col(COL_ISTA_SEG, kp_step(p, j, nullptr, j + 1 < L ? G.xw + (j + 1) * h : nullptr), s);
   }
-  (void)g;
   return e;
 }
 
 // Reverse steps L-1 .. 0 of one segment (g holds dL/dx at its end).
 cudaError_t enqueue_reverse(cs_plan_s* p, int L, cudaStream_t s) {
+  auto& G = p->gr;
+  const size_t h = (size_t)p->n / 2;
   cudaError_t e = cudaSuccess;
   for (int j = L - 1; j >= 0 && e == cudaSuccess; --j) {
-    e = launch_col(COL_GRAD_W, kp_step(p, j, 0), s);
-    if (e == cudaSuccess) e = launch_mid(MID_FWD, kp_step(p, j, 0), s);
-    if (e == cudaSuccess) e = launch_col(COL_GRAD_MASK, kp_step(p, j, 0), s);
-    if (e == cudaSuccess) e = launch_mid(MID_ADJ, kp_step(p, j, 0), s);
-    if (e == cudaSuccess) e = launch_col(COL_GRAD_G, kp_step(p, j, 0), s);
-    if (e == cudaSuccess) e = launch_col(COL_LOAD2, kp_step(p, j, 0), s);
-    if (e == cudaSuccess) e = launch_mid(MID_CORR, kp_step(p, j, 0), s);
-    if (e == cudaSuccess) e = launch_col(COL_LOAD2, kp_step(p, j, FL_PAIR2), s);
-    if (e == cudaSuccess) e = launch_mid(MID_CORR, kp_step(p, j, FL_PAIR2), s);
+    e = launch_col(j == L - 1 ? COL_GRAD_W : COL_GRAD_GW, kp_step(p, j), s);
+    if (e == cudaSuccess) e = launch_mid(MID_FWD_CORR, kp_step(p, j, nullptr, nullptr, G.rw + j * h), s);
+    if (e == cudaSuccess) e = launch_col(COL_GRAD_MASK, kp_step(p, j), s);
+    if (e == cudaSuccess) e = launch_mid(MID_ADJ_CORR, kp_step(p, j, nullptr, nullptr, G.xw + j * h), s);
   }
-  return e;
+  return e == cudaSuccess ? launch_col(COL_GRAD_G, kp_step(p, 0), s) : e;
 }
 
 }  // namespace
@@ -1223,21 +1228,20 @@ cs_status cs_grad(cs_plan_t p, const float* y, float lambda, float tau, int T, i
   p->ista_args = false;
   p->admm_args = false;
 
-  // per-step arguments of a segment
-  for (int j = 0; j <= K; ++j) {
-    CallArgs b{};
-    b.x = G.seg + j * n;
-    b.z = G.seg + (j + 1) * n;
-    b.v = G.rseg + j * n;
-    b.mu = G.w;
-    b.nu = G.q;
-    b.dst = j < K ? G.g : dc;   // entry K: the output pass (dL/dc, natural order)
-    b.aux = G.dy;
-    b.thr = thr;
-    b.tau = tau;
-    CS_TRY(launch_set_args(b, G.ca + j, s));
-  }
-  p->launches += K + 1;
+  // per-step arguments of a segment (one launch, as K of them took longer
+  // than a step), and entry K: the output pass (dL/dc, natural order)
+  CallArgs b{};
+  b.x = G.seg;
+  b.z = G.seg + n;
+  b.mu = G.w;
+  b.dst = G.g;
+  b.aux = G.dy;
+  b.thr = thr;
+  b.tau = tau;
+  CS_TRY(launch_set_args_seq(b, SEQ_X | SEQ_Z, (int64_t)n, K, G.ca, s));
+  b.dst = dc;
+  CS_TRY(launch_set_args(b, G.ca + K, s));
+  p->launches += 2;
   CS_TRY(launch_to_tile(gx_T, G.g, p->gi, 1, s));
   CS_TRY(cudaMemsetAsync(G.gacc, 0, tab_count(p->gi) * sizeof(float4), s));
   CS_TRY(cudaMemsetAsync(G.gpart, 0, p->gi.col_ctas * sizeof(double), s));
@@ -1250,12 +1254,12 @@ cs_status cs_grad(cs_plan_t p, const float* y, float lambda, float tau, int T, i
     CS_TRY(cudaMemcpyAsync(G.seg, G.ckpt + sg * n, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
     CS_TRY(run_graph(p, (uint64_t(3) << 40) | (uint32_t)L, [&](cudaStream_t st) { return enqueue_replay(p, L, st); }));
     CS_TRY(run_graph(p, (uint64_t(4) << 40) | (uint32_t)L, [&](cudaStream_t st) { return enqueue_reverse(p, L, st); }));
-    p->launches += 1 + 4 * L + 9 * L;
+    p->launches += 1 + 4 * L + 4 * L + 1;
   }
 
   // outputs: dL/dc from its spectrum, dL/dlambda = tau dL/dtheta, dL/dy by row
-  CS_TRY(launch_mid(MID_FROM_ACC, kp_step(p, K, 0), s));
-  CS_TRY(launch_col(COL_STORE, kp_step(p, K, 0), s));
+  CS_TRY(launch_mid(MID_FROM_ACC, kp_step(p, K), s));
+  CS_TRY(launch_col(COL_STORE, kp_step(p, K), s));
   CS_TRY(launch_sum_scaled(G.gpart, p->gi.col_ctas, tau, dlambda, s));
   CS_TRY(launch_gather_rows(G.dy, p->si.pos, p->m, dy, s));
   p->launches += 4;
@@ -1306,10 +1310,11 @@ cudaError_t grad_admm_reserve(cs_plan_s* p, int ck, int seg) {
 
 // Pass parameters of the ADMM gradient: the complex-n geometry, the reverse
 // exchange buffer and accumulators, and the CallArgs entry `ca`.
-KParams kp_admm(const cs_plan_s* p, const CallArgs* ca, float2* W, const float2* W2) {
+KParams kp_admm(const cs_plan_s* p, const CallArgs* ca, const float2* in, float2* W, const float2* W2) {
   KParams k = kparams(p, p->ga, 0);
+  k.pp.Wi = in;
   k.pp.W = W;
-  k.pp.W2 = const_cast<float2*>(W2);
+  k.pp.W2 = W2;
   k.pp.gacc_a = p->ga_.gacc;
   k.pp.gpart = p->ga_.gpart;
   k.ca = ca;
@@ -1317,18 +1322,17 @@ KParams kp_admm(const cs_plan_s* p, const CallArgs* ca, float2* W, const float2*
 }
 
 // Replay of one segment of L iterations from the state in (av, az, amu, anu):
-// iteration j keeps the column transform of its forward pair (wseg[j]) and
-// its soft-threshold input (sseg[j]).
+// iteration j's forward pair is transformed into wseg[j], where its mid pass
+// reads it and the reverse finds it, and its soft-threshold input is kept
+// (sseg[j]).
 cudaError_t enqueue_admm_replay(cs_plan_s* p, int L, cudaStream_t s) {
   auto& G = p->ga_;
   const size_t n = (size_t)p->n;
-  cudaError_t e = launch_col(COL_ADMM_INIT, kp_admm(p, G.ca, p->W, nullptr), s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(G.wseg, p->W, n * sizeof(float2), cudaMemcpyDeviceToDevice, s);
+  cudaError_t e = launch_col(COL_ADMM_INIT, kp_admm(p, G.ca, p->W, G.wseg, nullptr), s);
   for (int j = 0; j < L && e == cudaSuccess; ++j) {
-    e = launch_mid(MID_ADMM, kp_admm(p, G.ca + j, p->W, nullptr), s);
-    if (e == cudaSuccess) e = launch_col(COL_ADMM_SEG, kp_admm(p, G.ca + j, p->W, nullptr), s);
-    if (e == cudaSuccess && j + 1 < L)
-      e = cudaMemcpyAsync(G.wseg + (j + 1) * n, p->W, n * sizeof(float2), cudaMemcpyDeviceToDevice, s);
+    e = launch_mid(MID_ADMM, kp_admm(p, G.ca + j, G.wseg + j * n, p->W, nullptr), s);
+    if (e == cudaSuccess)
+      e = launch_col(COL_ADMM_SEG, kp_admm(p, G.ca + j, p->W, j + 1 < L ? G.wseg + (j + 1) * n : p->W, nullptr), s);
   }
   return e;
 }
@@ -1342,8 +1346,8 @@ cudaError_t enqueue_admm_reverse(cs_plan_s* p, int L, bool first, cudaStream_t s
   cudaError_t e = cudaSuccess;
   for (int j = L - 1; j >= 0 && e == cudaSuccess; --j) {
     const CallArgs* ca = (first && j == L - 1) ? G.ca + 2 * K : G.ca + K + j;
-    e = launch_col(COL_ADMM_REV, kp_admm(p, ca, G.Wr, nullptr), s);
-    if (e == cudaSuccess) e = launch_mid(MID_ADMM_REV, kp_admm(p, G.ca + K + j, G.Wr, G.wseg + j * n), s);
+    e = launch_col(COL_ADMM_REV, kp_admm(p, ca, G.Wr, G.Wr, nullptr), s);
+    if (e == cudaSuccess) e = launch_mid(MID_ADMM_REV, kp_admm(p, G.ca + K + j, G.Wr, G.Wr, G.wseg + j * n), s);
   }
   return e;
 }
@@ -1400,27 +1404,16 @@ extern "C" cs_status cs_grad_admm(cs_plan_t p, const float* y, float lambda, con
 
   // per-iteration arguments: replay (state in the plan's buffers), reverse,
   // the reverse of iteration T-1 (with dL/dz(T), dL/dx(T)), the output pass
-  for (int j = 0; j < Kc; ++j) {
-    CallArgs r = a;
-    r.x = nullptr;
-    r.aux = G.sseg + j * n;
-    CS_TRY(launch_set_args(r, G.ca + j, s));
-    CallArgs b = a;
-    b.x = nullptr;
-    b.z = nullptr;
-    b.mu = G.mub;
-    b.nu = G.nub;
-    b.v = G.dy;
-    b.aux = G.sseg + j * n;
-    CS_TRY(launch_set_args(b, G.ca + Kc + j, s));
-  }
   {
     CallArgs b = a;
     b.x = nullptr;
+    b.aux = G.sseg;
+    CS_TRY(launch_set_args_seq(b, SEQ_AUX, (int64_t)n, Kc, G.ca, s));
     b.z = nullptr;
     b.mu = G.mub;
     b.nu = G.nub;
     b.v = G.dy;
+    CS_TRY(launch_set_args_seq(b, SEQ_AUX, (int64_t)n, Kc, G.ca + Kc, s));
     const int jl = (T - (S - 1) * K) - 1;   // last iteration of the last segment
     b.aux = G.sseg + jl * n;
     b.src = G.gz;
@@ -1430,7 +1423,7 @@ extern "C" cs_status cs_grad_admm(cs_plan_t p, const float* y, float lambda, con
     o.dst = dc;
     CS_TRY(launch_set_args(o, G.ca + 2 * Kc + 1, s));
   }
-  p->launches += 2 * Kc + 2;
+  p->launches += 4;
   CS_TRY(launch_to_tile(gz_T, G.gz, p->ga, 0, s));
   if (gx_T) CS_TRY(launch_to_tile(gx_T, G.gx, p->ga, 0, s));
   CS_TRY(cudaMemsetAsync(G.mub, 0, nb, s));
@@ -1455,8 +1448,8 @@ extern "C" cs_status cs_grad_admm(cs_plan_t p, const float* y, float lambda, con
   }
 
   // outputs: dL/dc from its spectrum, dL/dlambda = sum / sigma, dL/dy by row
-  CS_TRY(launch_mid(MID_ADMM_FROM_ACC, kp_admm(p, G.ca + 2 * Kc + 1, G.Wr, nullptr), s));
-  CS_TRY(launch_col(COL_STORE_RE, kp_admm(p, G.ca + 2 * Kc + 1, G.Wr, nullptr), s));
+  CS_TRY(launch_mid(MID_ADMM_FROM_ACC, kp_admm(p, G.ca + 2 * Kc + 1, G.Wr, G.Wr, nullptr), s));
+  CS_TRY(launch_col(COL_STORE_RE, kp_admm(p, G.ca + 2 * Kc + 1, G.Wr, G.Wr, nullptr), s));
   CS_TRY(launch_sum_scaled(G.gpart, p->ga.col_ctas, (float)(1.0 / prm->sigma), dlambda, s));
   CS_TRY(launch_gather_rows(G.dy, p->sa.pos, p->m, dy, s));
   p->launches += 4;

@@ -11,6 +11,18 @@ constexpr int AUX_NT = 256;
 
 __global__ void set_args_k(CallArgs a, CallArgs* dst) { *dst = a; }
 
+// Arguments of a sequence of steps: entry j is `a` with the pointers named in
+// `adv` moved on by j * stride floats.
+__global__ void set_args_seq_k(CallArgs a, int adv, int64_t stride, int count, CallArgs* dst) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= count) return;
+  const int64_t o = (int64_t)j * stride;
+  if (adv & SEQ_X) a.x += o;
+  if (adv & SEQ_Z) a.z += o;
+  if (adv & SEQ_AUX) a.aux += o;
+  dst[j] = a;
+}
+
 // Deterministic final sum of per-block partials, slot by slot.
 __global__ void __launch_bounds__(AUX_NT) finalize_k(const double* __restrict__ partials, int nblk,
                                                      double* __restrict__ stats) {
@@ -378,6 +390,11 @@ inline unsigned blocks_for(int64_t count) { return (unsigned)((count + AUX_NT - 
 
 cudaError_t launch_set_args(const CallArgs& a, CallArgs* dst, cudaStream_t s) {
   set_args_k<<<1, 1, 0, s>>>(a, dst);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_set_args_seq(const CallArgs& a, int adv, int64_t stride, int count, CallArgs* dst, cudaStream_t s) {
+  set_args_seq_k<<<blocks_for(count), AUX_NT, 0, s>>>(a, adv, stride, count, dst);
   return cudaGetLastError();
 }
 

@@ -151,7 +151,8 @@ __device__ __forceinline__ void col_body(const KParams& kp, const int blk) {
   }
   pdl_wait();                                   // everything below may depend on earlier kernels
   const CallArgs a = *kp.ca;
-  float2* __restrict__ W = kp.pp.W;
+  float2* W = kp.pp.W;
+  const float2* Wi = kp.pp.Wi;   // may be W
   Acc acc;
   acc.zero();
   acc.smask = smask;
@@ -173,11 +174,11 @@ __device__ __forceinline__ void col_body(const KParams& kp, const int blk) {
         hook.q[i * R + r] = E::load(kp, a, col0 + vec + (idx << g.lgN1), (col0 << lgN2) + (idx << lgG) + vec, acc);
       }
     }
-    tile_fft<+1, TILE, NT, TWS>(sm, lay, tw, lgN2, hook, ColIO{W, col0, g.lgN1}, SmemIO{});
+    tile_fft<+1, TILE, NT, TWS>(sm, lay, tw, lgN2, hook, ColIO{const_cast<float2*>(Wi), col0, g.lgN1}, SmemIO{});
   } else if constexpr (E::kRead && SHAPE != 0) {
     // static shapes: the first inverse stage reads the exchange buffer itself
     EpiHook<KIND> hook{kp, a, col0, g.lgN1, acc, col0 << lgN2, lgG};
-    tile_fft<+1, TILE, NT, TWS>(sm, lay, tw, lgN2, hook, ColIO{W, col0, g.lgN1}, SmemIO{});
+    tile_fft<+1, TILE, NT, TWS>(sm, lay, tw, lgN2, hook, ColIO{const_cast<float2*>(Wi), col0, g.lgN1}, SmemIO{});
   } else if constexpr (E::kRead) {
     float4 buf[NLD];
 #pragma unroll
@@ -185,7 +186,7 @@ __device__ __forceinline__ void col_body(const KParams& kp, const int blk) {
       const int e = 2 * (threadIdx.x + i * NT);
       if (e < tot) {
         const int j2 = e >> lgG, c = e & (G - 1);
-        buf[i] = __ldcg(reinterpret_cast<const float4*>(W + col0 + c + ((size_t)j2 << g.lgN1)));
+        buf[i] = __ldcg(reinterpret_cast<const float4*>(Wi + col0 + c + ((size_t)j2 << g.lgN1)));
       }
     }
 #pragma unroll
@@ -206,7 +207,7 @@ __device__ __forceinline__ void col_body(const KParams& kp, const int blk) {
     }
     __syncthreads();
   }
-  if constexpr (KIND == COL_GRAD_W || KIND == COL_ADMM_REV) block_accum<NT>(acc.v[0], kp.pp.gpart, blk);
+  if constexpr (KIND == COL_GRAD_W || KIND == COL_GRAD_GW || KIND == COL_ADMM_REV) block_accum<NT>(acc.v[0], kp.pp.gpart, blk);
   if (kp.flags & FL_STATS) {
     constexpr int kSlots =
         KIND == COL_RESIDUAL ? (1 << ST_R2)
@@ -235,24 +236,6 @@ __device__ __forceinline__ void col_body(const KParams& kp, const int blk) {
       }
     }
   }
-  if constexpr (KIND == COL_LOAD2) {
-    // the second vector of the pair, to the second exchange buffer
-    __syncthreads();
-    for (int e = threadIdx.x; e < tot; e += NT) sm[pad(e)] = Epi<COL_LOAD2>::apply2(kp, a, (col0 << lgN2) + e);
-    __syncthreads();
-    tile_fft<-1, TILE, NT, TWS>(sm, lay, tw, lgN2);
-    float2* __restrict__ W2 = kp.pp.W2;
-#pragma unroll
-    for (int i = 0; i < NLD; ++i) {
-      const int e = 2 * (threadIdx.x + i * NT);
-      if (e < tot) {
-        const int j2 = e >> lgG, c = e & (G - 1);
-        const float2 lo = sm[pad(e)], hi = sm[pad(e + 1)];
-        __stcg(reinterpret_cast<float4*>(W2 + col0 + c + ((size_t)j2 << g.lgN1)),
-               make_float4(lo.x, lo.y, hi.x, hi.y));
-      }
-    }
-  }
 }
 
 template <int KIND, int SHAPE>
@@ -271,7 +254,7 @@ __global__ void __launch_bounds__(ColTile<SHAPE>::kTile / ColTile<SHAPE>::kVpt, 
 #define CS_COL_KINDS(X, S)                                                                     \
   X(COL_LOAD, S) X(COL_LOAD_SCALED, S) X(COL_STORE, S) X(COL_MASK, S) X(COL_RESIDUAL, S)         \
   X(COL_ISTA, S) X(COL_ISTA_LAST, S) X(COL_POWER_OUT, S) X(COL_ADMM_INIT, S) X(COL_ADMM, S)       \
-  X(COL_ADMM_LAST, S) X(COL_LOADT, S) X(COL_RES_SAVE, S) X(COL_ISTA_SEG, S) X(COL_GRAD_W, S)           \
-  X(COL_GRAD_MASK, S) X(COL_GRAD_G, S) X(COL_LOAD2, S) X(COL_ADMM_SEG, S) X(COL_ADMM_REV, S) X(COL_STORE_RE, S)
+  X(COL_ADMM_LAST, S) X(COL_LOADT, S) X(COL_ISTA_SEG, S) X(COL_GRAD_W, S)           \
+  X(COL_GRAD_MASK, S) X(COL_GRAD_G, S) X(COL_GRAD_GW, S) X(COL_ADMM_SEG, S) X(COL_ADMM_REV, S) X(COL_STORE_RE, S)
 
 }  // namespace csk

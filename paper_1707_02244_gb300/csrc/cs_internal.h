@@ -46,6 +46,7 @@ enum : int {
 
 // Plan-constant device pointers, passed by value to every pass kernel.
 struct PlanPtrs {
+  const float2* Wi;          // exchange buffer a pass reads (W unless a pass keeps its input)
   float2* W;                 // exchange buffer, complex[n]
   const uint32_t* mask;      // rows of Omega, one bit per row in tile order, [n/32]
   const uint32_t* prefix;    // set bits before word w, [n/32]
@@ -57,7 +58,7 @@ struct PlanPtrs {
   const float* tab_admm_b;   // 1 / (n (rho |chat_k|^2 + sigma)) per pair slot
   int* status;               // device status word
   // unrolled-ISTA gradient (cs_grad) only
-  float2* W2;                // second exchange buffer, complex[N] of the real-FFT geometry
+  const float2* W2;          // column transform of the vector a reverse mid pass correlates with
   float4* gacc;              // per pair slot: accumulated spectrum at (k, k + N)
   double* gpart;             // per column CTA: accumulated dL/dtheta
   // unrolled-ADMM gradient (cs_grad_admm) only
@@ -89,7 +90,7 @@ struct KParams {
   int flags;
 };
 
-enum : int { FL_STATS = 1, FL_WRITE_STATE = 2, FL_POWER_SCALE = 4, FL_PAIR2 = 8 };
+enum : int { FL_STATS = 1, FL_WRITE_STATE = 2, FL_POWER_SCALE = 4 };
 
 // Column-pass epilogues and mid-pass spectrum operators.
 enum ColKind : int {
@@ -106,12 +107,11 @@ enum ColKind : int {
   COL_ADMM_LAST,       // same without the forward FFT
   // unrolled-ISTA gradient (real-FFT geometry, vectors in tile order)
   COL_LOADT,           // forward FFT of x (tile order)
-  COL_RES_SAVE,        // as COL_RESIDUAL, and r -> v
   COL_ISTA_SEG,        // inverse, z <- eta(x + tau g) (x kept), forward
   COL_GRAD_W,          // w = dst on the support of z -> mu, dtheta partials, forward
-  COL_GRAD_MASK,       // inverse, q = M C w -> nu, aux += tau P C w, forward
+  COL_GRAD_MASK,       // inverse, q = M C w, aux += tau P C w, forward
   COL_GRAD_G,          // inverse, dst = mu - tau C^T q
-  COL_LOAD2,           // forward FFTs of (v, mu) -> (W, W2); with FL_PAIR2 of (nu, x)
+  COL_GRAD_GW,         // COL_GRAD_G of one step and COL_GRAD_W of the one before it
   // unrolled-ADMM gradient (complex-n geometry, vectors in tile order)
   COL_ADMM_SEG,        // as COL_ADMM (no state written), and s = x + nu -> aux
   COL_ADMM_REV,        // inverse (b' + i C b'), reverse of one Algorithm 3 iteration, forward FFT of (p' + i x')
@@ -119,7 +119,8 @@ enum ColKind : int {
 };
 enum MidKind : int {
   MID_FWD = 0, MID_ADJ, MID_ADMM,
-  MID_CORR,            // forward FFTs of W and W2 -> gacc += s conj(a^) b^ (s = -1 with FL_PAIR2)
+  MID_FWD_CORR,        // MID_FWD of w, and gacc += conj(r^) w^ with r's column transform in W2
+  MID_ADJ_CORR,        // MID_ADJ of q, and gacc -= conj(q^) x^ with x's in W2
   MID_FROM_ACC,        // tau / N times the packed spectrum of gacc -> inverse FFT -> W
   // unrolled-ADMM gradient (complex-n geometry)
   MID_ADMM_REV,        // FFTs of W (p' + i x') and W2 (the forward pair): b' = B (C^T p' + x'), dL/dc spectrum
@@ -145,6 +146,8 @@ cudaError_t init_multi_kernels(const Geo& g);
 
 // Small kernels (cs_aux.cu).
 cudaError_t launch_set_args(const CallArgs& a, CallArgs* dst, cudaStream_t s);
+enum : int { SEQ_X = 1, SEQ_Z = 2, SEQ_AUX = 4 };
+cudaError_t launch_set_args_seq(const CallArgs& a, int adv, int64_t stride, int count, CallArgs* dst, cudaStream_t s);
 cudaError_t launch_finalize(const double* partials, int nblk, double* stats, cudaStream_t s);
 cudaError_t launch_twiddle(float2* dst, int count, int64_t M, cudaStream_t s);
 cudaError_t launch_fft64(const double* c, double2* a, double2* b, int64_t n, double2** out,

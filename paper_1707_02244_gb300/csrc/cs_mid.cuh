@@ -196,7 +196,8 @@ __device__ __forceinline__ void mid_body(const KParams& kp, const int blk) {
   const int lgN1 = S::lgN1(g), N1 = 1 << lgN1;
   const int tot = (2 * U) << lgN1;
   const auto lay = S::lay(g);
-  float2* __restrict__ W = kp.pp.W;
+  float2* W = kp.pp.W;
+  const float2* Wi = kp.pp.Wi;   // may be W
   constexpr bool TWS = S::Lay::kStatic;   // static shape: twiddles in shared memory
   constexpr bool TWOD = S::kTwoD;         // 2D DFT: no four-step twiddle hooks
   constexpr int LGN1S = TWS ? S::lgN1(Geo{}) : 4;
@@ -304,7 +305,7 @@ __device__ __forceinline__ void mid_body(const KParams& kp, const int blk) {
   }
   pdl_wait();   // everything above reads plan constants; W is not one
   const float a_rho = kp.ca->rho, a_sigma = kp.ca->sigma;   // ADMM only
-  auto load_tile = [&](float2* dst, const float2* __restrict__ src) {
+  auto load_tile = [&](float2* dst, const float2* src) {
     float4 buf[NLD];
 #pragma unroll
     for (int i = 0; i < NLD; ++i) {
@@ -330,7 +331,7 @@ __device__ __forceinline__ void mid_body(const KParams& kp, const int blk) {
   auto fwd_rows_from_global = [&]() {
     if constexpr (TWS) {
       __syncthreads();
-      const MidIO io{W, u0, lgN1, g.N2};
+      const MidIO io{const_cast<float2*>(Wi), u0, lgN1, g.N2};
       if constexpr (TWOD) {
         NoHook nh;
         tile_fft<-1, TILE, NT, true>(sm, lay, tws, lgN1, nh, io, SmemIO{});
@@ -352,22 +353,29 @@ __device__ __forceinline__ void mid_body(const KParams& kp, const int blk) {
       tile_fft<-1, TILE, NT, false>(buf, lay, g.tw1, lgN1 + 1, h);
     }
   };
-  if constexpr (KIND == MID_CORR) {
-    // Spectra of two packed real vectors a (W) and b (W2).  From the pair
-    // (Z_k, Z_{N-k}) of a packed spectrum: E = (Z_k + conj Z_{N-k}) / 2,
+  if constexpr (KIND == MID_FWD_CORR || KIND == MID_ADJ_CORR) {
+    // The product of the vector in W (as MID_FWD, MID_ADJ) and its correlation
+    // with the vector in W2, both packed real.  From the pair (Z_k, Z_{N-k})
+    // of a packed spectrum: E = (Z_k + conj Z_{N-k}) / 2,
     // O = (Z_k - conj Z_{N-k}) / 2i, and the length-2N real spectrum is
     // a^_k = E + w O, a^_{k+N} = E - w O, w = exp(-2 pi i k / 2N).
+    constexpr bool ADJ = KIND == MID_ADJ_CORR;
     float2* sm2 = sm + smem_slots(TILE);
-    load_tile(sm, W);
-    fwd_rows(sm);
     load_tile(sm2, kp.pp.W2);
     fwd_rows(sm2);
-    const float sgn = (kp.flags & FL_PAIR2) ? -1.f : 1.f;
+    if constexpr (TWS) {
+      fwd_rows_from_global();
+    } else {
+      load_tile(sm, Wi);
+      fwd_rows(sm);
+    }
     for (int t = threadIdx.x; t < nslots; t += NT) {
       int ea, eb, k2, k1, tidx;
       slot_at(t, ea, eb, k2, k1, tidx);
-      const float2 w = cmul(__ldg(g.twr + k2), __ldg(g.tw1 + k1));
-      float2 sa[2], sb[2];
+      const float2 w = phase_at(k2, k1);
+      const float4 tab = __ldg(kp.pp.tab_ista + tidx);
+      float4 acc = kp.pp.gacc[tidx];
+      float2 sp[2][2];   // [W, W2][k, k + N]
 #pragma unroll
       for (int v = 0; v < 2; ++v) {
         const float2* bufv = v ? sm2 : sm;
@@ -375,19 +383,24 @@ __device__ __forceinline__ void mid_body(const KParams& kp, const int blk) {
         const float2 E = make_float2(0.5f * (za.x + zb.x), 0.5f * (za.y - zb.y));
         const float2 O = make_float2(0.5f * (za.y + zb.y), -0.5f * (za.x - zb.x));
         const float2 wo = cmul(w, O);
-        float2* dst = v ? sb : sa;
-        dst[0] = cadd(E, wo);
-        dst[1] = csub(E, wo);
+        sp[v][0] = cadd(E, wo);
+        sp[v][1] = csub(E, wo);
       }
-      const float2 p0 = cmulc(sb[0], sa[0]), p1 = cmulc(sb[1], sa[1]);   // conj(a^) b^
-      float4 acc = kp.pp.gacc[tidx];
+      // + conj(r^) w^ (W: w, W2: r), - conj(q^) x^ (W: q, W2: x)
+      const float sgn = ADJ ? -1.f : 1.f;
+      const float2 p0 = ADJ ? cmulc(sp[1][0], sp[0][0]) : cmulc(sp[0][0], sp[1][0]);
+      const float2 p1 = ADJ ? cmulc(sp[1][1], sp[0][1]) : cmulc(sp[0][1], sp[1][1]);
       acc.x = fmaf(sgn, p0.x, acc.x);
       acc.y = fmaf(sgn, p0.y, acc.y);
       acc.z = fmaf(sgn, p1.x, acc.z);
       acc.w = fmaf(sgn, p1.y, acc.w);
       kp.pp.gacc[tidx] = acc;
+      float2 za = sm[pad(ea)], zb = sm[pad(eb)];
+      op_real<ADJ>(tab, w, za, zb);
+      sm[pad(eb)] = zb;   // self-pairs (ea == eb) keep the k-side value
+      sm[pad(ea)] = za;
     }
-    return;
+    __syncthreads();
   } else if constexpr (KIND == MID_ADMM_REV) {
     // Reverse of the x-update of one Algorithm 3 iteration.  W holds the
     // column transform of p' + i x', W2 that of the iteration's forward pair
@@ -401,7 +414,7 @@ __device__ __forceinline__ void mid_body(const KParams& kp, const int blk) {
     // pairs C x with b' and C b' with x, whose sum is real times chat), and
     // Bs + i conj(chat) Bs goes back for the inverse: b' + i C b'.
     float2* sm2 = sm + smem_slots(TILE);
-    load_tile(sm, W);
+    load_tile(sm, Wi);
     fwd_rows(sm);
     load_tile(sm2, kp.pp.W2);
     fwd_rows(sm2);
@@ -467,7 +480,7 @@ __device__ __forceinline__ void mid_body(const KParams& kp, const int blk) {
     if constexpr (TWS) {
       fwd_rows_from_global();
     } else {
-      load_tile(sm, W);
+      load_tile(sm, Wi);
       fwd_rows(sm);
     }
     // spectrum operator over all (k, N-k) pairs held by this CTA (unrolled so
@@ -541,11 +554,13 @@ __global__ void __launch_bounds__(Cfg<TILE, MidShape<SHAPE>::kVpt>::NT, Cfg<TILE
 }  // namespace
 
 #define CS_MID_KINDS(X, T, S)                                                                    \
-  X(MID_FWD, T, S) X(MID_ADJ, T, S) X(MID_ADMM, T, S) X(MID_CORR, T, S) X(MID_FROM_ACC, T, S)       \
+  X(MID_FWD, T, S) X(MID_ADJ, T, S) X(MID_ADMM, T, S) X(MID_FWD_CORR, T, S) X(MID_ADJ_CORR, T, S) X(MID_FROM_ACC, T, S)       \
   X(MID_ADMM_REV, T, S) X(MID_ADMM_FROM_ACC, T, S)
 #define CS_MID_KINDS_2D(X, T, S) X(MID_FWD, T, S) X(MID_ADJ, T, S) X(MID_ADMM, T, S)
 
-// MID_CORR and MID_ADMM_REV hold two tiles in shared memory
-constexpr int mid_smem_mult(int kind) { return (kind == MID_CORR || kind == MID_ADMM_REV) ? 2 : 1; }
+// the reverse passes that correlate hold two tiles in shared memory
+constexpr int mid_smem_mult(int kind) {
+  return (kind == MID_FWD_CORR || kind == MID_ADJ_CORR || kind == MID_ADMM_REV) ? 2 : 1;
+}
 
 }  // namespace csk

@@ -98,7 +98,7 @@ struct RowSel {
 // Which epilogues look up the row mask, and how many mask bits one element
 // of the tile holds (2 in the packed real-FFT geometry, 1 in complex-n).
 template <int KIND> struct UsesMask {
-  static constexpr int kBits = (KIND == COL_RESIDUAL || KIND == COL_MASK || KIND == COL_RES_SAVE ||
+  static constexpr int kBits = (KIND == COL_RESIDUAL || KIND == COL_MASK ||
                                 KIND == COL_GRAD_MASK) ? 2
                               : (KIND == COL_ADMM || KIND == COL_ADMM_LAST || KIND == COL_ADMM_SEG ||
                                  KIND == COL_ADMM_REV) ? 1 : 0;
@@ -395,26 +395,18 @@ template <> struct Epi<COL_ADMM_REV> {
 // exactly when |u(t)| > theta, and then sign u(t) = sign x(t+1)):
 //   dL/dx(t) = w - tau C^T M C w,  dL/dtheta += -sum sign(x(t+1)) w,
 //   dL/dy += tau P C w,  dL/dc_k += tau sum_i (r_i w_{i+k} - q_i x(t)_{i+k})
-// with q = M C w.  CallArgs of one step: x = x(t), z = x(t+1), v = r(t),
-// mu = w, nu = q, dst = g, aux = dL/dy (compact, tile order of the rows); all
-// n-vectors packed float2 in tile order.
+// with q = M C w.  CallArgs of one step: x = x(t), z = x(t+1), mu = w,
+// dst = g, aux = dL/dy (compact, tile order of the rows); all n-vectors packed
+// float2 in tile order.  The two correlations want the spectra of r, w, q and
+// x(t): w and q pass through the mid passes of C w and C^T q anyway, and the
+// column transforms of r and x(t) are what the replay's passes wrote, kept
+// instead of the vectors.  So a step is reversed in 4 passes (9 when the four
+// transforms were formed again for the correlations).
 
 template <> struct Epi<COL_LOADT> {
   static constexpr bool kRead = false, kFwd = true;
   __device__ static float2 apply(const KParams&, const CallArgs& a, float2, int p, int t, Acc&) {
     return ld2(a.x, t);
-  }
-};
-
-template <> struct Epi<COL_RES_SAVE> : EpiRows2 {
-  static constexpr bool kRead = true, kFwd = true;
-  __device__ static float2 apply(const KParams& kp, const CallArgs& a, float2 v, int p, int t, Acc& acc,
-                                 const Pre& q) {
-    const float r0 = (q.mm & 1u) ? q.y0 - v.x : 0.f;
-    const float r1 = (q.mm & 2u) ? q.y1 - v.y : 0.f;
-    const float2 r = make_float2(r0, r1);
-    st2(a.v, t, r);
-    return r;
   }
 };
 
@@ -450,9 +442,7 @@ template <> struct Epi<COL_GRAD_MASK> {
     // each compact row index belongs to one element: plain read-modify-write
     if (mm & 1u) a.aux[i0] = fmaf(a.tau, v.x, a.aux[i0]);
     if (mm & 2u) a.aux[i0 + (int)(mm & 1u)] = fmaf(a.tau, v.y, a.aux[i0 + (int)(mm & 1u)]);
-    const float2 q = make_float2((mm & 1u) ? v.x : 0.f, (mm & 2u) ? v.y : 0.f);
-    st2(a.nu, t, q);
-    return q;
+    return make_float2((mm & 1u) ? v.x : 0.f, (mm & 2u) ? v.y : 0.f);   // q
   }
 };
 
@@ -466,14 +456,19 @@ template <> struct Epi<COL_GRAD_G> {
   }
 };
 
-// (r, w) -> (W, W2); with FL_PAIR2 (q, x(t)) -> (W, W2)
-template <> struct Epi<COL_LOAD2> {
-  static constexpr bool kRead = false, kFwd = true;
-  __device__ static float2 apply(const KParams& kp, const CallArgs& a, float2, int p, int t, Acc&) {
-    return ld2((kp.flags & FL_PAIR2) ? a.nu : a.v, t);
+// g of the step reversed before (its w is in mu), and this step's w in its place
+template <> struct Epi<COL_GRAD_GW> {
+  static constexpr bool kRead = true, kFwd = true;
+  struct Pre { float2 w, x; };
+  __device__ static Pre load(const KParams&, const CallArgs& a, int p, int t, const Acc&) {
+    return Pre{ld2(a.mu, t), ld2(a.z, t)};
   }
-  __device__ static float2 apply2(const KParams& kp, const CallArgs& a, int t) {
-    return ld2((kp.flags & FL_PAIR2) ? a.x : a.mu, t);
+  __device__ static float2 apply(const KParams&, const CallArgs& a, float2 v, int p, int t, Acc& acc, const Pre& q) {
+    const float2 g = make_float2(fmaf(-a.tau, v.x, q.w.x), fmaf(-a.tau, v.y, q.w.y));
+    const float2 w = make_float2(q.x.x != 0.f ? g.x : 0.f, q.x.y != 0.f ? g.y : 0.f);
+    acc.v[0] -= sgnf(q.x.x) * w.x + sgnf(q.x.y) * w.y;
+    st2(a.mu, t, w);
+    return w;
   }
 };
 
