@@ -296,7 +296,7 @@ __device__ __forceinline__ void mid_body(const KParams& kp, const int blk) {
       slot_at(threadIdx.x + i * NT, ea, eb, k2, k1, tidx);
       if constexpr (KIND == MID_ADMM) {
         pw[i] = __ldg(kp.pp.tab_admm_c + tidx);
-        pt[i].x = __ldg(kp.pp.tab_admm_b + tidx);
+        pt[i].x = __ldcg(kp.pp.tab_admm_b + tidx);   // re-tabulated between calls
       } else {
         pt[i] = __ldg(kp.pp.tab_ista + tidx);
         pw[i] = phase_at(k2, k1);

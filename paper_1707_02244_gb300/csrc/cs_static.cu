@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kColNt) static_fwd_k(const double* __restrict_
 }
 
 // Launch 2: rows (u, N2 - u), or 0 and N2/2 for u = 0.
-__global__ void __launch_bounds__(kMidNt) static_mid_k(double2* __restrict__ w, int lgN1, int lgN2, int transpose) {
+__global__ void __launch_bounds__(kMidNt) static_mid_k(double2* w, int lgN1, int lgN2, int transpose) {
   __shared__ double2 rt[2 * kRoots], A[4 * kRoots / 2], B[4 * kRoots / 2];   // N1 <= 64
   dep_trigger();
   const int N1 = 1 << lgN1, N2 = 1 << lgN2, lgN = lgN1 + lgN2, u = blockIdx.x;
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(kMidNt) static_mid_k(double2* __restrict__ w, 
   // vectors 0, 1: the rows of c; 2, 3: of x
   for (int t = threadIdx.x; t < 4 << lgN1; t += kMidNt) {
     const int v = t >> lgN1, q = t & (N1 - 1);
-    A[t] = w[((int64_t)(v >> 1) << lgN) + ((int64_t)row[v & 1] << lgN1) + q];
+    A[t] = __ldcg(w + ((int64_t)(v >> 1) << lgN) + ((int64_t)row[v & 1] << lgN1) + q);
   }
   double2* r = fft64_tile<-1>(A, B, lgN1, 4, rt);
   double2* o = r == A ? B : A;
@@ -301,14 +301,15 @@ __global__ void __launch_bounds__(kMidNt) static_mid_k(double2* __restrict__ w, 
 }
 
 // Launch 3: column blockIdx.x of the result.
-__global__ void __launch_bounds__(kColNt) static_inv_k(const double2* __restrict__ w, float* __restrict__ y, int lgN1,
-                                                       int lgN2) {
+// (w is read through L2: a read-only load could be moved above the wait for
+// the launch that writes it)
+__global__ void __launch_bounds__(kColNt) static_inv_k(const double2* w, float* __restrict__ y, int lgN1, int lgN2) {
   __shared__ double2 rt[2 * kRoots], A[kRoots], B[kRoots];
   dep_trigger();
   const int N2 = 1 << lgN2, j1 = blockIdx.x;
   load_roots(rt);
   dep_wait();
-  for (int k2 = threadIdx.x; k2 < N2; k2 += kColNt) A[k2] = w[(k2 << lgN1) + j1];
+  for (int k2 = threadIdx.x; k2 < N2; k2 += kColNt) A[k2] = __ldcg(w + (k2 << lgN1) + j1);
   const double2* r = fft64_tile<+1>(A, B, lgN2, 1, rt);
   for (int j2 = threadIdx.x; j2 < N2; j2 += kColNt) {
     const int p = j1 + (j2 << lgN1);
