@@ -223,13 +223,13 @@ cs_status cs_grad_admm(cs_plan_t plan, const float* y, float lambda, const cs_ad
  * for many independent instances at once).  Instance i has its own n_i,
  * m_i, rows and c.  Three solvers share a call:
  *   - power-of-two n_i <= CS_BATCH_MAX_N: one CTA per instance, the iterate
- *     kept in shared memory for all iterations (one launch per size class,
+ *     kept on chip for all iterations (one launch per size class,
  *     on up to 4 internal streams forked from the batch's stream);
  *   - larger power-of-two n_i: the buffers and tables of a plan, iterated
  *     together (every pass of an iteration is one launch over the tiles of
- *     all of them; their whole solve is one CUDA graph launch);
+ *     all instances of one length; their whole solve is one CUDA graph launch);
  *   - 7-smooth n_i = 2^a 3^b 5^c 7^d that is not a power of two: mixed-radix
- *     FFTs (radices 8, 4, 2, 7, 5, 3), one CTA per instance up to n_i = 4096,
+ *     FFTs (radices 2 to 10), one CTA per instance up to n_i = 4096,
  *     above it a four-step split n_i = N1 N2 chosen by a plan-time tuner
  *     (cached per n for the process; CS_BATCH_AUTOTUNE=0 in the
  *     environment keeps the heuristic split; CS_BATCH_TUNE_CACHE=<file>
