@@ -166,7 +166,8 @@ void make_geo(Geo& g, int lgN, bool small_tiles) {
 
 // 2D DFT of an N2 x N1 array (2^lgN2 rows of 2^lgN1): the same two passes
 // without the four-step twiddle.  Column pass: 4096-value tiles while
-// N2 <= 2048, 8192-value tiles of two columns for N2 = 4096.
+// N2 <= 1024, tiles of four columns (a full 32-byte sector of every row) for
+// N2 = 2048 and 4096.
 void make_geo2d(Geo& g, int lgN2, int lgN1) {
   g.lgN = lgN2 + lgN1;
   g.N = 1 << g.lgN;
@@ -174,7 +175,7 @@ void make_geo2d(Geo& g, int lgN2, int lgN1) {
   g.N2 = 1 << lgN2;
   g.lgN1 = lgN1;
   g.N1 = 1 << lgN1;
-  const int lgCol = lgN2 <= 11 ? 12 : 14;
+  const int lgCol = lgN2 <= 10 ? 12 : lgN2 == 11 ? 13 : 14;
   g.col_tile = 1 << lgCol;
   g.lgG = (lgCol - lgN2) < lgN1 ? (lgCol - lgN2) : lgN1;
   g.G = 1 << g.lgG;
@@ -200,7 +201,8 @@ bool geo_ok(const Geo& g) {
   if (g.twod)
     return g.N2 >= 2 && g.N1 >= 2 && g.G >= 2 && g.col_ctas >= 1 && g.mid_ctas >= 1 && g.U >= 1 &&
            2 * g.U <= 64 && (2 * g.U) * g.N1 <= g.tile && (g.G << g.lgN2) <= g.col_tile && g.N1 <= 4096 &&
-           (g.col_tile == 4096 || g.col_r8 || (g.lgN2 == 12 && g.lgG == 2 && g.col_tile == 16384));
+           (g.col_tile == 4096 || g.col_r8 || (g.lgN2 == 11 && g.lgG == 2 && g.col_tile == 8192) ||
+            (g.lgN2 == 12 && g.lgG == 2 && g.col_tile == 16384));
   return g.N1 >= g.N2 && g.N2 >= 2 && g.G >= 2 && g.col_ctas >= 1 && g.mid_ctas >= 1 &&
          2 * g.U <= 64 && (2 * g.U) * g.N1 <= g.tile && (g.G << g.lgN2) <= 4096;
 }

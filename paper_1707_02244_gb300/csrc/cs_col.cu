@@ -11,6 +11,8 @@ cudaError_t init_col_kernels(const Geo& g) {
   if (e == cudaSuccess) e = set_smem(col_kernel<k, S>, ColTile<S>::kTile, ColTile<S>::kMinB);
   if (g.col_tile == COL_TILE4) {
     CS_COL_KINDS_2D(CS_SET_COL, 3)
+  } else if (g.col_tile == COL_TILE2) {
+    CS_COL_KINDS_2D(CS_SET_COL, 5)
   } else if (g.lgN2 == 10 && g.lgG == 2) {
     CS_COL_KINDS(CS_SET_COL, 1)
   } else {
@@ -29,6 +31,10 @@ cudaError_t launch_col(ColKind kind, const KParams& kp, cudaStream_t s) {
   if (g.col_tile == COL_TILE4) {
     if (g.lgN2 == 12 && g.lgG == 2) {
       switch (kind) { CS_COL_KINDS_2D(CS_L_COL, 3) default: break; }
+    }
+  } else if (g.col_tile == COL_TILE2) {
+    if (g.lgN2 == 11 && g.lgG == 2) {
+      switch (kind) { CS_COL_KINDS_2D(CS_L_COL, 5) default: break; }
     }
   } else if (hot) {
     switch (kind) { CS_COL_KINDS(CS_L_COL, 1) }
