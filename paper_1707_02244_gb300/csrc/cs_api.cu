@@ -71,6 +71,7 @@ struct cs_plan_s {
     float* tb = nullptr;
   } sml;
   bool cluster_i = false, cluster_a = false;   // one cluster solves the instance
+  float2 *twn_i = nullptr, *twn_a = nullptr;   // its four-step twiddles, exp(-2 pi i q / N)
   CallArgs last_ca{};              // arguments of the last single-CTA solve: cs_profile_pass sends them first
   bool ca_stale = false;
   // unrolled-ISTA gradient (cs_grad): allocated at the first call, grown on demand
@@ -162,6 +163,11 @@ void make_geo(Geo& g, int lgN, bool small_tiles) {
     r8_col(g);
     r8_mid(g);
   }
+  // The 4096- and 8192-value shapes of N >= 2^20 form most stage twiddles as
+  // products (fewer shared-memory reads: their passes are bound by that pipe);
+  // every other shape reads each twiddle as a value rounded once.
+  g.tw1_full = g.mid_r8 || !small_tiles;
+  g.tw2_full = g.col_r8 || !small_tiles;
 }
 
 // 2D DFT of an N2 x N1 array (2^lgN2 rows of 2^lgN1): the same two passes
@@ -194,6 +200,8 @@ void make_geo2d(Geo& g, int lgN2, int lgN1) {
   g.col_r8 = g.mid_r8 = 0;
   if (lgN2 >= 5 && lgN2 <= 9 && lgN1 >= (lgN2 == 5 ? 3 : 2)) r8_col(g);
   if (lgN1 >= 6 && lgN1 <= 10 && lgN2 >= 3) r8_mid(g);
+  g.tw1_full = g.mid_r8;                  // as make_geo: not the rows of 2048 and 4096 ...
+  g.tw2_full = g.col_r8 || lgN2 == 11;    // ... nor the columns of 1024 and 4096
 }
 
 // Geometry invariants the pass kernels rely on (checked for every plan).
@@ -234,7 +242,8 @@ void free_plan(cs_plan_s* p) {
                   p->dense, p->dense2, p->dense3};
   for (void* b : bufs)
     if (b) cudaFree(b);
-  void* sbufs[] = {p->sml.tA, p->sml.tB, p->sml.tc, p->sml.tw_i, p->sml.tw_a, p->sml.abs2, p->sml.tb};
+  void* sbufs[] = {p->sml.tA, p->sml.tB, p->sml.tc, p->sml.tw_i, p->sml.tw_a, p->sml.abs2, p->sml.tb,
+                   p->twn_i, p->twn_a};
   for (void* b : sbufs)
     if (b) cudaFree(b);
   void* gbufs[] = {p->gr.ckpt, p->gr.seg, p->gr.rw, p->gr.xw, p->gr.g, p->gr.w, p->gr.dy, p->gr.gacc,
@@ -291,8 +300,8 @@ cudaError_t make_tables(Geo& g, float2* base, cudaStream_t s) {
   if (e == cudaSuccess) e = launch_twiddle(twl, g.N1, g.N, s);
   if (e == cudaSuccess) e = launch_twiddle(twr, g.N2, 2 * (int64_t)g.N, s);
   if (e == cudaSuccess) e = launch_twiddle(tw1h, g.N1, g.N1, s);
-  if (e == cudaSuccess) e = launch_stage_tw(tws1, g.lgN1, g.mid_r8 ? 3 : 4, s);
-  if (e == cudaSuccess) e = launch_stage_tw(tws2, g.lgN2, g.col_r8 ? 3 : 4, s);
+  if (e == cudaSuccess) e = launch_stage_tw(tws1, g.lgN1, g.mid_r8 ? 3 : 4, g.tw1_full, s);
+  if (e == cudaSuccess) e = launch_stage_tw(tws2, g.lgN2, g.col_r8 ? 3 : 4, g.tw2_full, s);
   g.tw1 = tw1;
   g.tw2 = tw2;
   g.twl = twl;
@@ -459,6 +468,7 @@ SmallArgs small_args(const cs_plan_s* p, bool admm) {
 ClusterArgs cluster_args(const cs_plan_s* p, bool admm) {
   ClusterArgs a{};
   a.geo = admm ? p->ga : p->gi;
+  a.twn = admm ? p->twn_a : p->twn_i;
   const cs_plan_s::Sel& sel = admm ? p->sa : p->si;
   a.mask = sel.mask;
   a.prefix = sel.prefix;
@@ -647,19 +657,27 @@ cs_status build_plan(cs_plan_t* out, int64_t n0, int64_t n1, int64_t m, const in
   if (p->small_i) {
     CS_PLAN_TRY(dalloc(&p->sml.tA, n / 4 + 1));
     CS_PLAN_TRY(dalloc(&p->sml.tB, n / 4 + 1));
-    CS_PLAN_TRY(dalloc(&p->sml.tw_i, small_tw_count(lgn - 1)));
+    CS_PLAN_TRY(dalloc(&p->sml.tw_i, small_tw_count(lgn - 1, false)));
     if (p->small_a) {
       CS_PLAN_TRY(dalloc(&p->sml.tc, n / 2 + 1));
       CS_PLAN_TRY(dalloc(&p->sml.abs2, n / 2 + 1));
       CS_PLAN_TRY(dalloc(&p->sml.tb, n / 2 + 1));
-      CS_PLAN_TRY(dalloc(&p->sml.tw_a, small_tw_count(lgn)));
+      CS_PLAN_TRY(dalloc(&p->sml.tw_a, small_tw_count(lgn, false)));
     }
     CS_PLAN_TRY(launch_small_tables(chat, n, p->sml.tA, p->sml.tB, p->sml.tc, p->sml.abs2, s));
-    CS_PLAN_TRY(launch_small_tw(lgn - 1, p->sml.tw_i, s));
-    if (p->small_a) CS_PLAN_TRY(launch_small_tw(lgn, p->sml.tw_a, s));
+    CS_PLAN_TRY(launch_small_tw(lgn - 1, false, p->sml.tw_i, s));
+    if (p->small_a) CS_PLAN_TRY(launch_small_tw(lgn, false, p->sml.tw_a, s));
   }
   p->cluster_i = !p->small_i && small_tiles && cluster_init(p->gi, false);
   p->cluster_a = !p->small_a && small_tiles && cluster_init(p->ga, true);
+  if (p->cluster_i) {
+    CS_PLAN_TRY(dalloc(&p->twn_i, p->gi.N));
+    CS_PLAN_TRY(launch_twiddle(p->twn_i, p->gi.N, p->gi.N, s));
+  }
+  if (p->cluster_a) {
+    CS_PLAN_TRY(dalloc(&p->twn_a, p->ga.N));
+    CS_PLAN_TRY(launch_twiddle(p->twn_a, p->ga.N, p->ga.N, s));
+  }
   CS_PLAN_TRY(admm_table(p, 1.0, 1.0, s, nullptr));
   CS_PLAN_TRY(launch_build_mask(d_rows, m, n, p->gi, 1, p->si.mask, p->status, s));
   CS_PLAN_TRY(launch_build_mask(d_rows, m, n, p->ga, 0, p->sa.mask, p->status, s));

@@ -54,15 +54,15 @@ __global__ void twiddle_k(float2* dst, int count, int64_t M) {
 // Stage-major twiddle table of a length-L FFT (see stage_twiddle): the
 // stage with span Ls and radix R holds w_{Ls R}^(r k) at row(r) Ls + k for
 // the rows r it keeps (tw_row_r).
-__global__ void stage_tw_k(float2* dst, int lgL, int lgRmax, int count) {
+__global__ void stage_tw_k(float2* dst, int lgL, int lgRmax, bool full, int count) {
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= count) return;
   int lgLs = lgRmax;
   while (true) {
     const int lgR = (lgL - lgLs) >= lgRmax ? lgRmax : (lgL - lgLs);
-    const int sz = tw_rows(lgR) << lgLs;
+    const int sz = tw_rows(lgR, full) << lgLs;
     if (t < sz) {
-      const int r = tw_row_r(lgR, t >> lgLs), k = t & ((1 << lgLs) - 1);
+      const int r = tw_row_r(lgR, t >> lgLs, full), k = t & ((1 << lgLs) - 1);
       double sn, cs;
       sincospi(-2.0 * (double)(r * k) / (double)(1 << (lgLs + lgR)), &sn, &cs);
       dst[blockIdx.x * blockDim.x + threadIdx.x] = make_float2((float)cs, (float)sn);
@@ -459,9 +459,9 @@ cudaError_t launch_tab_ista(const double2* chat, const Geo& g, int64_t n, float4
   return cudaGetLastError();
 }
 
-cudaError_t launch_stage_tw(float2* dst, int lgL, int lgRmax, cudaStream_t s) {
-  const int count = stage_tw_count(lgL, lgRmax);
-  if (count > 0) stage_tw_k<<<blocks_for(count), AUX_NT, 0, s>>>(dst, lgL, lgRmax, count);
+cudaError_t launch_stage_tw(float2* dst, int lgL, int lgRmax, bool full, cudaStream_t s) {
+  const int count = stage_tw_count(lgL, lgRmax, full);
+  if (count > 0) stage_tw_k<<<blocks_for(count), AUX_NT, 0, s>>>(dst, lgL, lgRmax, full, count);
   return cudaGetLastError();
 }
 

@@ -435,7 +435,7 @@ cs_status cs_batch_plan(cs_batch_t* out, int count, const int64_t* n, const int6
     int64_t twn = 0;
     for (int i : b->small)
       for (int lg : {hd[i].lgn - 1, hd[i].lgn})
-        if (twoff.emplace(lg, twn).second) twn += (small_tw_count(lg) + 1) & ~1;
+        if (twoff.emplace(lg, twn).second) twn += (small_tw_count(lg, true) + 1) & ~1;
     const int ns = (int)b->small.size();
     int64_t ms = 0;
     for (int i : b->small) ms += m[i];
@@ -455,7 +455,7 @@ cs_status cs_batch_plan(cs_batch_t* out, int count, const int64_t* n, const int6
     CS_B_TRY(balloc(&b->status, 1));
     CS_B_TRY(cudaMemsetAsync(b->status, 0, sizeof(int), s));
     CS_B_TRY(cudaMemcpyAsync(b->descs, hd.data(), count * sizeof(BatchDesc), cudaMemcpyHostToDevice, s));
-    for (const auto& kv : twoff) CS_B_TRY(launch_small_tw(kv.first, b->tw + kv.second, s));
+    for (const auto& kv : twoff) CS_B_TRY(launch_small_tw(kv.first, true, b->tw + kv.second, s));
     std::vector<SmallInst> hs_inst(ns);
     ms = 0;
     for (int k = 0; k < ns; ++k) {

@@ -34,7 +34,7 @@ template <int LGN> struct ClShape {
   using ColLay = LoopLayout<StaticLayout<kLgN2, kLgG, true, 3>>;
   using RowLay = LoopLayout<StaticLayout<kLgN1, kLgRows, false, 3>>;
   static constexpr int kLob = kLgN1 - 3 < 4 ? kLgN1 - 3 : 4;
-  static constexpr int kTw1 = stage_tw_count(kLgN1, 3), kTw2 = stage_tw_count(kLgN2, 3);
+  static constexpr int kTw1 = stage_tw_count(kLgN1, 3, true), kTw2 = stage_tw_count(kLgN2, 3, true);
   static constexpr int kLo = 1 << kLob, kHi = 1 << (kLgN1 - kLob);
   static constexpr int kLohi = (1 << kLgRows) * (kLo + kHi);
   // float2 of dynamic shared memory: FFT scratch, row and column inputs, tables
@@ -129,8 +129,9 @@ template <int LGN> struct ClCtx {
 };
 
 template <int LGN>
-__device__ __forceinline__ ClCtx<LGN> cl_begin(const Geo& g, float2* base) {
+__device__ __forceinline__ ClCtx<LGN> cl_begin(const ClusterArgs& a, float2* base) {
   using S = ClShape<LGN>;
+  const Geo& g = a.geo;
   __shared__ int zero;
   if (threadIdx.x == 0) zero = 0;   // read behind the first barrier
   ClCtx<LGN> x;
@@ -152,7 +153,10 @@ __device__ __forceinline__ ClCtx<LGN> cl_begin(const Geo& g, float2* base) {
     const int vec = is_lo ? tt / S::kLo : tt / S::kHi;
     const int q = is_lo ? tt % S::kLo : (tt % S::kHi) << S::kLob;
     const int slot = (x.rank << S::kLgRows) + vec;
-    x.lohi[t] = tw4(g, (q * slot_row(g, slot >> 1, slot & 1)) & (g.N - 1));
+    // one rounded value (the passes' tw4 is a product of two): the 128-point
+    // transforms have a stage more here than radix 16 gives them, and with tw4
+    // an ADMM solve at n = 2^14, 2^15 rounded 3 % more than by the passes
+    x.lohi[t] = __ldg(a.twn + ((q * slot_row(g, slot >> 1, slot & 1)) & (g.N - 1)));
   }
   return x;
 }
@@ -271,7 +275,7 @@ template <int LGN>
 __global__ void __launch_bounds__(ClShape<LGN>::NT, 1) cluster_ista_k(const ClusterArgs a) {
   using S = ClShape<LGN>;
   extern __shared__ float2 smem[];
-  const ClCtx<LGN> x = cl_begin<LGN>(a.geo, smem);
+  const ClCtx<LGN> x = cl_begin<LGN>(a, smem);
   ClOpReal<LGN> tab;
   tab.load(a, x.rank);
   // the thread's elements: x, the kept rows' y
@@ -347,7 +351,7 @@ template <int LGN>
 __global__ void __launch_bounds__(ClShape<LGN>::NT, 1) cluster_admm_k(const ClusterArgs a) {
   using S = ClShape<LGN>;
   extern __shared__ float2 smem[];
-  const ClCtx<LGN> x = cl_begin<LGN>(a.geo, smem);
+  const ClCtx<LGN> x = cl_begin<LGN>(a, smem);
   float2 tc[4];
   float tb[4];
 #pragma unroll
@@ -429,7 +433,7 @@ __global__ void __launch_bounds__(ClShape<LGN>::NT, 1) cluster_power_k(const Clu
   using S = ClShape<LGN>;
   extern __shared__ float2 smem[];
   __shared__ double red[S::NT / 32][2], part[CL][2], tot[2];
-  const ClCtx<LGN> x = cl_begin<LGN>(a.geo, smem);
+  const ClCtx<LGN> x = cl_begin<LGN>(a, smem);
   ClOpReal<LGN> tab;
   tab.load(a, x.rank);
   float2 w[VPT8], u[VPT8];
@@ -519,7 +523,7 @@ __global__ void __launch_bounds__(ClShape<LGN>::NT, 1) cluster_power_k(const Clu
 template <int LGN, bool ADJ>
 __global__ void __launch_bounds__(ClShape<LGN>::NT, 1) cluster_product_k(const ClusterArgs a) {
   extern __shared__ float2 smem[];
-  const ClCtx<LGN> x = cl_begin<LGN>(a.geo, smem);
+  const ClCtx<LGN> x = cl_begin<LGN>(a, smem);
   ClOpReal<LGN> tab;
   tab.load(a, x.rank);
   const float2* src = reinterpret_cast<const float2*>(a.x);

@@ -64,10 +64,10 @@ struct EpiHook {
 // G = 4 columns, the geometry of every N >= 2^20, fixed at compile time.
 // SHAPE 10 + LGN2 (LGN2 = 5 .. 9): radix-8 tiles of 4 columns (8 for
 // LGN2 = 5), 8 values per thread.
-// SHAPE 40 + LGN2 (LGN2 = 6 .. 9): 4096-value tiles, 16 values per thread
+// SHAPE 40 + LGN2 (LGN2 = 6 .. 10): 4096-value tiles, 16 values per thread
 // (grouped launches).
 template <int SHAPE> struct ColShape {
-  static_assert((SHAPE >= 15 && SHAPE <= 19) || (SHAPE >= 46 && SHAPE <= 49), "column shapes");
+  static_assert((SHAPE >= 15 && SHAPE <= 19) || (SHAPE >= 46 && SHAPE <= 50), "column shapes");
   static constexpr bool kR8 = SHAPE < 40;
   static constexpr int kLgN2 = SHAPE % (kR8 ? 10 : 40), kLgG = kR8 ? (kLgN2 == 5 ? 3 : 2) : 12 - kLgN2;
   using Lay = StaticLayout<kLgN2, kLgG, true, kR8 ? 3 : 4>;
@@ -82,7 +82,7 @@ template <> struct ColShape<0> {
   __device__ static int lgN2(const Geo& g) { return g.lgN2; }
 };
 template <> struct ColShape<1> {
-  using Lay = StaticLayout<10, 2, true>;
+  using Lay = StaticLayout<10, 2, true, 4, false>;
   __device__ static Lay lay(const Geo&) { return Lay{}; }
   __device__ static constexpr int lgG(const Geo&) { return 2; }
   __device__ static constexpr int lgN2(const Geo&) { return 10; }
@@ -90,7 +90,7 @@ template <> struct ColShape<1> {
 
 // SHAPE 3: N2 = 4096 and G = 4, 16384-value tiles (1024 threads).
 template <> struct ColShape<3> {
-  using Lay = StaticLayout<12, 2, true>;
+  using Lay = StaticLayout<12, 2, true, 4, false>;
   __device__ static Lay lay(const Geo&) { return Lay{}; }
   __device__ static constexpr int lgG(const Geo&) { return 2; }
   __device__ static constexpr int lgN2(const Geo&) { return 12; }
@@ -127,6 +127,7 @@ template <int SHAPE> struct ColTile {
   static constexpr int kMinB = kR8 ? Cfg<kTile, kVpt>::MINB : SHAPE == 3 ? COL_MINB4 : SHAPE == 5 ? COL_MINB2 : COL_MINB;
   static constexpr int kCarve = kR8 ? 0 : kMinB;
   static constexpr int kLgR = kR8 ? 3 : 4;
+  static constexpr bool kTwFull = SHAPE != 1 && SHAPE != 3;   // as the shape's layout
 };
 
 // The column pass of tile `blk` (columns blk G .. blk G + G - 1).
@@ -146,7 +147,7 @@ __device__ __forceinline__ void col_body(const KParams& kp, const int blk) {
   const int tot = G << lgN2;
   const auto lay = S::lay(g);
   constexpr bool TWS = SHAPE != 0;   // static shape: stage-major twiddles in shared memory
-  constexpr int TW_N = TWS ? stage_tw_count(ColTile<SHAPE>::kLgN2, ColTile<SHAPE>::kLgR) : 2;
+  constexpr int TW_N = TWS ? stage_tw_count(ColTile<SHAPE>::kLgN2, ColTile<SHAPE>::kLgR, ColTile<SHAPE>::kTwFull) : 2;
   __shared__ __align__(16) float2 tws[TW_N];
   const float2* tw = TWS ? tws : g.tw2;
   if (TWS) copy_table<NT>(tws, g.tws2, TW_N);   // plan constant

@@ -137,10 +137,11 @@ struct DynLayout {
   }
 };
 
-// LGR: log2 of the leading radix (4: 16 values per thread, 3: 8).
-template <int LGL, int LGNV, bool VEC_FAST, int LGR = 4>
+// LGR: log2 of the leading radix (4: 16 values per thread, 3: 8).  TWF: the
+// stage tables hold every twiddle (see stage_twiddle).
+template <int LGL, int LGNV, bool VEC_FAST, int LGR = 4, bool TWF = true>
 struct StaticLayout {
-  static constexpr bool kStatic = true;
+  static constexpr bool kStatic = true, kTwFull = TWF;
   static constexpr int kLgL = LGL, kLgNv = LGNV, kLgR = LGR;
   __device__ __forceinline__ constexpr int LG() const { return LGL; }
   __device__ __forceinline__ constexpr int NV() const { return LGNV; }
@@ -198,29 +199,37 @@ struct SmemIO {
 };
 
 // Stage-major twiddle tables keep, for a stage of span Ls and radix R, the
-// rows r of w_{Ls R}^(r k) (k < Ls) that stage_twiddle reads: r = 1, 2, 3, 4,
-// 8, 12 for radix 16, r = 1 .. 4 for radix 8, r = 1 .. R-1 for radix 4 and 2.
-// Row `row` of a stage holds r = tw_row_r(lgR, row).
-__host__ __device__ constexpr int tw_rows(int lgR) { return lgR == 4 ? 6 : lgR == 3 ? 4 : lgR == 2 ? 3 : 1; }
-__host__ __device__ constexpr int tw_row_r(int lgR, int row) { return lgR == 4 && row >= 4 ? 4 * (row - 2) : row + 1; }
+// rows r of w_{Ls R}^(r k) (k < Ls) that stage_twiddle reads: all of r = 1 ..
+// R-1 (FULL), or r = 1, 2, 3, 4, 8, 12 for radix 16 and r = 1 .. 4 for radix 8.
+// Row `row` of a stage holds r = tw_row_r(lgR, row, full).
+__host__ __device__ constexpr int tw_rows(int lgR, bool full) {
+  return full ? (1 << lgR) - 1 : lgR == 4 ? 6 : lgR == 3 ? 4 : lgR == 2 ? 3 : 1;
+}
+__host__ __device__ constexpr int tw_row_r(int lgR, int row, bool full) {
+  return !full && lgR == 4 && row >= 4 ? 4 * (row - 2) : row + 1;
+}
 __host__ __device__ constexpr int tw_row_of(int lgR, int r) { return lgR == 4 && r >= 8 ? r / 4 + 2 : r - 1; }
 
 // Multiply the R inputs of a butterfly by w^(r k), r = 1 .. R-1, from the
 // stage's block tw[row(r) Ls + k] = w^(r k) of the table in shared memory.
-// Radix 16 reads r = 1, 2, 3, 4, 8, 12 and forms the other nine as
-// w^((r1 + 4 r2) k) = w^(r1 k) w^(4 r2 k); radix 8 reads r = 1 .. 4 and forms
-// r = 5 .. 7 as w^(4k) w^((r - 4) k).  Every table value is an FP64 result
-// rounded once, so each twiddle is at most one product away from it; the
-// shared-memory reads drop from 15 to 6 (radix 16) and from 7 to 4 (radix 8).
-template <int R, int DIR>
+// Every table value is an FP64 result rounded once.  FULL: each twiddle is a
+// table value.  Otherwise radix 16 reads r = 1, 2, 3, 4, 8, 12 and forms the
+// other nine as w^((r1 + 4 r2) k) = w^(r1 k) w^(4 r2 k), radix 8 reads r = 1 ..
+// 4 and forms r = 5 .. 7 as w^(4k) w^((r - 4) k): 6 shared-memory reads in
+// place of 15 (4 in place of 7) for a twiddle that is a product of two rounded
+// values.
+template <int R, int DIR, bool FULL>
 __device__ __forceinline__ void stage_twiddle(float2* v, const float2* __restrict__ tw, int Ls, int k) {
   constexpr int lgR = R == 2 ? 1 : R == 4 ? 2 : R == 8 ? 3 : 4;
   auto get = [&](int r) {
-    float2 w = tw[tw_row_of(lgR, r) * Ls + k];
+    float2 w = tw[(FULL ? r - 1 : tw_row_of(lgR, r)) * Ls + k];
     if (DIR > 0) w.y = -w.y;
     return w;
   };
-  if constexpr (R == 16) {
+  if constexpr (FULL) {
+#pragma unroll
+    for (int r = 1; r < R; ++r) v[r] = cmul(v[r], get(r));
+  } else if constexpr (R == 16) {
     const float2 w1 = get(1), w2 = get(2), w3 = get(3);
     const float2 w4 = get(4), w8 = get(8), w12 = get(12);
     v[1] = cmul(v[1], w1);
@@ -317,7 +326,7 @@ __device__ __forceinline__ void stockham_stage(float2* s, const LAY& lay, int lg
       }
       if (!first) {
         if constexpr (TWS) {
-          stage_twiddle<R, DIR>(v[i], tw, Ls, k);
+          stage_twiddle<R, DIR, LAY::kTwFull>(v[i], tw, Ls, k);
         } else {
           const int kk = k << lgstep;   // w_{Ls R}^(r k) = tw[r * kk]
 #pragma unroll
@@ -373,7 +382,7 @@ __device__ __forceinline__ void tile_fft(float2* s, const LAY& lay, const float2
           stockham_stage<8, DIR, TILE, NT, TWS>(s, lay, 3 * st, tws, lgLt, hook, SmemIO{}, out);
         else
           stockham_stage<8, DIR, TILE, NT, TWS>(s, lay, 3 * st, tws, lgLt, hook);
-        if (st > 0) off8 += tw_rows(3) << (3 * st);
+        if (st > 0) off8 += tw_rows(3, LAY::kTwFull) << (3 * st);
       }
       const float2* tw8 = TWS ? tw + off8 : tw;
       if constexpr (rem8 == 2) stockham_stage<4, DIR, TILE, NT, TWS>(s, lay, LGL - 2, tw8, lgLt, hook, SmemIO{}, out);
@@ -394,7 +403,7 @@ __device__ __forceinline__ void tile_fft(float2* s, const LAY& lay, const float2
           stockham_stage<16, DIR, TILE, NT, TWS>(s, lay, 4 * st, tws, lgLt, hook, SmemIO{}, out);
         else
           stockham_stage<16, DIR, TILE, NT, TWS>(s, lay, 4 * st, tws, lgLt, hook);
-        if (st > 0) off += tw_rows(4) << (4 * st);
+        if (st > 0) off += tw_rows(4, LAY::kTwFull) << (4 * st);
       }
       const float2* twr = TWS ? tw + off : tw;
       if constexpr (rem == 3) stockham_stage<8, DIR, TILE, NT, TWS>(s, lay, LGL - 3, twr, lgLt, hook, SmemIO{}, out);
@@ -422,12 +431,12 @@ __device__ __forceinline__ void tile_fft(float2* s, const LAY& lay, const float2
 
 // Entries of the stage-major twiddle table of a length-L FFT: stage s >= 1
 // (span Ls, radix R) contributes tw_rows(log2 R) * Ls entries.  lgRmax: log2
-// of the leading radix.
-__host__ __device__ constexpr int stage_tw_count(int lgL, int lgRmax = 4) {
+// of the leading radix.  (`full` gives L - 2^lgRmax in all.)
+__host__ __device__ constexpr int stage_tw_count(int lgL, int lgRmax, bool full) {
   int n = 0, lgLs = 0;
   while (lgLs < lgL) {
     const int lgR = (lgL - lgLs) >= lgRmax ? lgRmax : (lgL - lgLs);
-    if (lgLs > 0) n += tw_rows(lgR) << lgLs;
+    if (lgLs > 0) n += tw_rows(lgR, full) << lgLs;
     lgLs += lgR;
   }
   return n;

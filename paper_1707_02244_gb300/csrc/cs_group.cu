@@ -55,8 +55,8 @@ cudaError_t launch_multi(K kern, int grid, const KParams* kps, const int2* map, 
   X(COL_LOAD, S) X(COL_RESIDUAL, S) X(COL_ISTA, S) X(COL_ISTA_LAST, S) X(COL_ADMM_INIT, S) X(COL_ADMM, S) \
   X(COL_ADMM_LAST, S)
 #define CS_MID_KINDS_MULTI(X, S) X(MID_FWD, S) X(MID_ADJ, S) X(MID_ADMM, S)
-#define CS_COL_SHAPES(X, K) X(6, K, 46) X(7, K, 47) X(8, K, 48) X(9, K, 49) X(10, K, 1)
-#define CS_MID_SHAPES(X, K) X(7, K, 57) X(8, K, 58) X(9, K, 59) X(10, K, 1) X(11, K, 2)
+#define CS_COL_SHAPES(X, K) X(6, K, 46) X(7, K, 47) X(8, K, 48) X(9, K, 49) X(10, K, 50)
+#define CS_MID_SHAPES(X, K) X(7, K, 57) X(8, K, 58) X(9, K, 59) X(10, K, 60) X(11, K, 61)
 
 bool multi_geo(const Geo& g) {
   return !g.twod && !g.col_r8 && !g.mid_r8 && g.tile == 4096 && g.col_tile == 4096 && g.lgN2 >= 6 && g.lgN2 <= 10 &&

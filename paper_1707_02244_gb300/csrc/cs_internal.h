@@ -22,6 +22,7 @@ struct Geo {
   int tile;            // mid pass: complex values per CTA; threads = tile / 16 (tile / 8 with mid_r8)
   int col_tile;        // column pass: complex values per CTA; threads = col_tile / 16 (/ 8 with col_r8)
   int col_r8, mid_r8;  // 1: the pass runs 8 values per thread and radix-8 stages (small tiles, see make_geo)
+  int tw1_full, tw2_full;   // 1: tws1 / tws2 hold every stage twiddle (see make_geo)
   int twod;            // 1: 2D DFT of the N2 x N1 array (no four-step twiddle; pairs (k2, k1) ~ (-k2, -k1))
   const float2* tw1;   // exp(-2 pi i q / (2 N1)), q < 2 N1
   const float2* tw2;   // exp(-2 pi i q / N2),     q < N2
@@ -164,7 +165,7 @@ cudaError_t launch_fft64_2d(const double* c2, double2* a, double2* b, int64_t n0
                             cudaStream_t s);
 // Pair slots of the mid pass (spectrum tables' length).
 inline int64_t tab_count(const Geo& g) { return ((int64_t)(g.N2 >> 1) << g.lgN1) + (g.twod ? 2 : 1); }
-cudaError_t launch_stage_tw(float2* dst, int lgL, int lgRmax, cudaStream_t s);
+cudaError_t launch_stage_tw(float2* dst, int lgL, int lgRmax, bool full, cudaStream_t s);
 cudaError_t launch_tab_admm(const double2* chat, const Geo& g, int64_t n, float2* tabc,
                             double* abs2, cudaStream_t s);
 cudaError_t launch_tab_admm_b(const double* abs2, int count, int64_t n, double rho,
@@ -218,8 +219,10 @@ struct SmallArgs {
   float thr, tau, rho, sigma, tau1, tau2, d_on, d_off;
 };
 cudaError_t launch_small(SmallKind kind, int lgN, const SmallArgs& a, cudaStream_t s);
-int small_tw_count(int lgN);
-cudaError_t launch_small_tw(int lgN, float2* tw, cudaStream_t s);   // small_tw_count(lgN) values
+// Stage twiddles, small_tw_count values: `full` for the size classes, else for
+// the solves and products of a plan (see SmallTw).
+int small_tw_count(int lgN, bool full);
+cudaError_t launch_small_tw(int lgN, bool full, float2* tw, cudaStream_t s);
 // Pair-operator tables of one instance from its FP64 spectrum: tA, tB n/4 + 1
 // values, tc, abs2 n/2 + 1 (null: no ADMM).
 cudaError_t launch_small_tables(const double2* chat, int64_t n, float4* tA, float2* tB, float2* tc, double* abs2,
@@ -248,6 +251,7 @@ cudaError_t launch_small_class(bool admm, int lgN, const SmallInst* inst, int co
 enum ClusterKind : int { CLUSTER_ISTA, CLUSTER_ADMM, CLUSTER_POWER, CLUSTER_FWD, CLUSTER_ADJ };
 struct ClusterArgs {
   Geo geo;
+  const float2* twn;               // exp(-2 pi i q / N), q < N
   const uint32_t *mask, *prefix;   // rows of Omega and compact y in the plan's tile order
   const float* ys;
   const float4* tab_i;

@@ -144,15 +144,16 @@ __device__ __forceinline__ void op_admm(const float2 ch, const float bb, float r
 // packed and the complex geometry of a 4096 x 4096 image.
 // SHAPE 10 + LGN1 (1D) and 30 + LGN1 (2D), LGN1 = 6 .. 10: radix-8 tiles of
 // one row pair (two for LGN1 = 6), 8 values per thread.
-// SHAPE 50 + LGN1 (1D, LGN1 = 7 .. 9): 4096-value tiles, 16 values per thread
+// SHAPE 50 + LGN1 (1D, LGN1 = 7 .. 11): 4096-value tiles, 16 values per thread
 // (grouped launches).
 template <int SHAPE> struct MidShape {
-  static_assert((SHAPE >= 16 && SHAPE <= 20) || (SHAPE >= 36 && SHAPE <= 40) || (SHAPE >= 57 && SHAPE <= 59),
+  static_assert((SHAPE >= 16 && SHAPE <= 20) || (SHAPE >= 36 && SHAPE <= 40) || (SHAPE >= 57 && SHAPE <= 61),
                 "mid shapes");
   static constexpr bool kTwoD = SHAPE >= 30 && SHAPE <= 40, kR8 = SHAPE < 50;
   static constexpr int kLgN1 = SHAPE - (kTwoD ? 30 : kR8 ? 10 : 50);
   static constexpr int kLgU = kR8 ? (kLgN1 == 6 ? 1 : 0) : 11 - kLgN1;
   static constexpr int kLgR = kR8 ? 3 : 4, kVpt = kR8 ? VPT8 : EPT;
+  static constexpr bool kTwFull = true;
   using Lay = StaticLayout<kLgN1, kLgU + 1, false, kLgR>;
   __device__ static Lay lay(const Geo&) { return Lay{}; }
   __device__ static constexpr int lgN1(const Geo&) { return kLgN1; }
@@ -160,15 +161,15 @@ template <int SHAPE> struct MidShape {
 };
 template <> struct MidShape<0> {
   using Lay = DynLayout;
-  static constexpr bool kTwoD = false;
+  static constexpr bool kTwoD = false, kTwFull = false;
   static constexpr int kLgR = 4, kVpt = EPT;
   __device__ static Lay lay(const Geo& g) { return Lay{g.lgN1, g.lgU + 1, false}; }
   __device__ static int lgN1(const Geo& g) { return g.lgN1; }
   __device__ static int lgU(const Geo& g) { return g.lgU; }
 };
 template <int LGN1, int LGU, bool TWOD = false> struct MidShapeS {
-  using Lay = StaticLayout<LGN1, LGU + 1, false>;
-  static constexpr bool kTwoD = TWOD;
+  using Lay = StaticLayout<LGN1, LGU + 1, false, 4, false>;
+  static constexpr bool kTwoD = TWOD, kTwFull = false;
   static constexpr int kLgR = 4, kVpt = EPT;
   __device__ static Lay lay(const Geo&) { return Lay{}; }
   __device__ static constexpr int lgN1(const Geo&) { return LGN1; }
@@ -203,7 +204,7 @@ __device__ __forceinline__ void mid_body(const KParams& kp, const int blk) {
   constexpr int LGN1S = TWS ? S::lgN1(Geo{}) : 4;
   constexpr int ROWS = TWS ? (2 << S::lgU(Geo{})) : MID_MAX_ROWS;
   constexpr int LOB = LGN1S - S::kLgR < 4 ? LGN1S - S::kLgR : 4;   // see MidTwHookS
-  constexpr int TW_N = TWS ? stage_tw_count(LGN1S, S::kLgR) : 2;
+  constexpr int TW_N = TWS ? stage_tw_count(LGN1S, S::kLgR, S::kTwFull) : 2;
   __shared__ __align__(16) float2 tws[TW_N];
   // static shapes: per-row lo[] and hi[]; dynamic: rt (see MidTwHook)
   constexpr int LOHI = (TWS && !TWOD) ? ROWS * ((1 << LOB) + (1 << (LGN1S - LOB))) : 2;

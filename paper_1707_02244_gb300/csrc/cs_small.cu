@@ -54,9 +54,9 @@ struct OpAdmm {
   }
 };
 
-template <int LG>
+template <int LG, bool FULL>
 __device__ __forceinline__ void load_tw(float2* dst, const float2* __restrict__ src) {
-  for (int i = threadIdx.x; i < SmallShape<LG>::kTw; i += SmallShape<LG>::NT) dst[i] = __ldg(src + i);
+  for (int i = threadIdx.x; i < SmallTw<LG, FULL>::kTw; i += SmallShape<LG>::NT) dst[i] = __ldg(src + i);
 }
 
 // Sum over the CTA in a fixed order; every thread gets it.
@@ -92,16 +92,16 @@ __device__ __forceinline__ void stage_y(const SmallArgs& a, int n, float* yd, ui
 
 // ISTA (Algorithm 1): n = 2 N packed, x (natural order, any 4-byte boundary)
 // in and out.
-template <int LG>
+template <int LG, bool FULL>
 __device__ __forceinline__ void small_ista(const SmallArgs& a) {
   using S = SmallShape<LG>;
   constexpr int N = S::N, E = S::E, ST = N / E, NT = S::NT;
   extern __shared__ float2 sm[];
   float2 *S0 = sm, *S1 = S0 + small_buf<LG>(), *tw = S1 + small_buf<LG>();
-  float2* yd = tw + ((S::kTw + 1) & ~1);
+  float2* yd = tw + ((SmallTw<LG, FULL>::kTw + 1) & ~1);
   __shared__ uint32_t mk[2 * N / 32];
   __shared__ double red[NT / 32];
-  load_tw<LG>(tw, a.tw);
+  load_tw<LG, FULL>(tw, a.tw);
   stage_y<NT>(a, 2 * N, reinterpret_cast<float*>(yd), mk);
   const int tid = threadIdx.x;
   const bool act = tid < S::NA;
@@ -123,7 +123,7 @@ __device__ __forceinline__ void small_ista(const SmallArgs& a) {
   for (int it = 0; it < a.iters; ++it) {
     const bool st = a.stats != nullptr && it + 1 == a.iters;
     float r2 = 0.f;
-    small_conv<LG>(v, S0, S1, tw, opf);
+    small_conv<LG, FULL>(v, S0, S1, tw, opf);
     if (act) {
 #pragma unroll
       for (int r = 0; r < E; ++r) {
@@ -134,7 +134,7 @@ __device__ __forceinline__ void small_ista(const SmallArgs& a) {
         v[r] = make_float2(r0, r1);
       }
     }
-    small_conv<LG>(v, S0, S1, tw, opa);
+    small_conv<LG, FULL>(v, S0, S1, tw, opa);
     float dx2 = 0.f, x2 = 0.f, l1 = 0.f, er = 0.f, nf = 0.f;
     if (act) {
 #pragma unroll
@@ -179,7 +179,7 @@ __device__ __forceinline__ void small_ista(const SmallArgs& a) {
 
 // Algorithm 3, n = N (complex): state (v, z, mu, nu) in natural order, in
 // when a.warm (else zero), out where the pointer is not null.
-template <int LG>
+template <int LG, bool FULL>
 __device__ __forceinline__ void small_admm(const SmallArgs& a) {
   using S = SmallShape<LG>;
   constexpr int N = S::N, E = S::E, ST = N / E, NT = S::NT;
@@ -188,7 +188,7 @@ __device__ __forceinline__ void small_admm(const SmallArgs& a) {
   float* yd = reinterpret_cast<float*>(S1);   // only until the registers hold it
   __shared__ uint32_t mk[N / 32];
   __shared__ double red[NT / 32];
-  load_tw<LG>(tw, a.tw);
+  load_tw<LG, FULL>(tw, a.tw);
   stage_y<NT>(a, N, yd, mk);
   const int tid = threadIdx.x;
   const bool act = tid < S::NA;
@@ -211,7 +211,7 @@ __device__ __forceinline__ void small_admm(const SmallArgs& a) {
   for (int it = 0; it < a.iters; ++it) {
     const bool end = it + 1 == a.iters, st = a.stats != nullptr && end;
     float r2 = 0.f, dx2 = 0.f, x2 = 0.f, l1 = 0.f, er = 0.f, nf = 0.f;
-    small_conv<LG>(v, S0, S1, tw, op);
+    small_conv<LG, FULL>(v, S0, S1, tw, op);
     if (act) {
 #pragma unroll
       for (int r = 0; r < E; ++r) {
@@ -259,9 +259,9 @@ __device__ __forceinline__ void small_admm(const SmallArgs& a) {
 }
 
 template <int LG>
-__global__ void __launch_bounds__(SmallShape<LG>::NT) small_ista_k(const SmallArgs a) { small_ista<LG>(a); }
+__global__ void __launch_bounds__(SmallShape<LG>::NT) small_ista_k(const SmallArgs a) { small_ista<LG, false>(a); }
 template <int LG>
-__global__ void __launch_bounds__(SmallShape<LG>::NT) small_admm_k(const SmallArgs a) { small_admm<LG>(a); }
+__global__ void __launch_bounds__(SmallShape<LG>::NT) small_admm_k(const SmallArgs a) { small_admm<LG, false>(a); }
 
 // Instance blockIdx.x of a size class of a batch: its constants, its scalars
 // of this call, and the call's concatenated vectors.
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(SmallShape<LG>::NT)
   d.tw = d.tw_i;
   SmallArgs a = class_args(d, sc[d.id], y, iters);
   a.x = x + d.noff;
-  small_ista<LG>(a);
+  small_ista<LG, true>(a);
 }
 template <int LG>
 __global__ void __launch_bounds__(SmallShape<LG>::NT)
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(SmallShape<LG>::NT)
   d.tw = d.tw_a;
   SmallArgs a = class_args(d, sc[d.id], y, iters);
   a.z = z + d.noff;
-  small_admm<LG>(a);
+  small_admm<LG, true>(a);
 }
 
 // Power iteration on A^T A from the fixed start vector in a.x (natural
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(SmallShape<LG>::NT) small_power_k(const SmallA
   float2 *S0 = sm, *S1 = S0 + small_buf<LG>(), *tw = S1 + small_buf<LG>();
   __shared__ uint32_t mk[2 * N / 32];
   __shared__ double red[NT / 32];
-  load_tw<LG>(tw, a.tw);
+  load_tw<LG, false>(tw, a.tw);
   for (int i = threadIdx.x; i < 2 * N / 32; i += NT) mk[i] = 0u;
   __syncthreads();
   for (int i = threadIdx.x; i < a.m; i += NT) {
@@ -350,11 +350,11 @@ __global__ void __launch_bounds__(SmallShape<LG>::NT) small_power_k(const SmallA
     const float s = (float)rsqrt(x2);
 #pragma unroll
     for (int r = 0; r < E; ++r) u[r] = v[r] = act ? cscale(v[r], s) : make_float2(0.f, 0.f);
-    small_conv<LG>(v, S0, S1, tw, opf);
+    small_conv<LG, false>(v, S0, S1, tw, opf);
 #pragma unroll
     for (int r = 0; r < E; ++r)
       v[r] = make_float2(((mb >> (2 * r)) & 1u) ? v[r].x : 0.f, ((mb >> (2 * r)) & 2u) ? v[r].y : 0.f);
-    small_conv<LG>(v, S0, S1, tw, opa);
+    small_conv<LG, false>(v, S0, S1, tw, opa);
     float n2 = 0.f, uw = 0.f;
     if (act) {
 #pragma unroll
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(SmallShape<LG>::NT) small_product_k(const Smal
   constexpr int N = S::N, E = S::E, ST = N / E, NT = S::NT;
   extern __shared__ float2 sm[];
   float2 *S0 = sm, *S1 = S0 + small_buf<LG>(), *tw = S1 + small_buf<LG>();
-  float2* d = tw + ((S::kTw + 1) & ~1);
+  float2* d = tw + ((SmallTw<LG, false>::kTw + 1) & ~1);
   const int tid = threadIdx.x;
   const bool act = tid < S::NA;
   float2 v[E];
@@ -390,8 +390,8 @@ __global__ void __launch_bounds__(SmallShape<LG>::NT) small_product_k(const Smal
 #pragma unroll
       for (int r = 0; r < E; ++r) v[r] = __ldg(xg + tid + r * ST);
     }
-    load_tw<LG>(tw, a.tw);   // read behind the product's first barrier
-    small_conv<LG>(v, S0, S1, tw, OpReal<false>{a.tA, a.tB});
+    load_tw<LG, false>(tw, a.tw);   // read behind the product's first barrier
+    small_conv<LG, false>(v, S0, S1, tw, OpReal<false>{a.tA, a.tB});
     if (act) {
 #pragma unroll
       for (int r = 0; r < E; ++r) d[tid + r * ST] = v[r];
@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(SmallShape<LG>::NT) small_product_k(const Smal
     const float* df = reinterpret_cast<const float*>(d);
     for (int i = tid; i < a.m; i += NT) a.yo[i] = df[__ldg(a.rows + i)];
   } else {
-    load_tw<LG>(tw, a.tw);
+    load_tw<LG, false>(tw, a.tw);
     for (int i = tid; i < N; i += NT) d[i] = make_float2(0.f, 0.f);
     __syncthreads();
     for (int i = tid; i < a.m; i += NT) reinterpret_cast<float*>(d)[__ldg(a.rows + i)] = __ldg(a.y + i);
@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(SmallShape<LG>::NT) small_product_k(const Smal
 #pragma unroll
       for (int r = 0; r < E; ++r) v[r] = d[tid + r * ST];
     }
-    small_conv<LG>(v, S0, S1, tw, OpReal<true>{a.tA, a.tB});
+    small_conv<LG, false>(v, S0, S1, tw, OpReal<true>{a.tA, a.tB});
     if (act) {
 #pragma unroll
       for (int r = 0; r < E; ++r) xg[tid + r * ST] = v[r];
@@ -424,7 +424,7 @@ __global__ void small_tw_k(float2* dst, SmallTwStages d) {
   if (t >= d.total) return;
   int b = 0;
   while (b + 1 < d.count && t >= d.off[b + 1]) ++b;
-  const int q = t - d.off[b], r = tw_row_r(d.lgR[b], q >> d.lgLs[b]), k = q & ((1 << d.lgLs[b]) - 1);
+  const int q = t - d.off[b], r = small_tw_r(d, b, q >> d.lgLs[b]), k = q & ((1 << d.lgLs[b]) - 1);
   double sn, cs;
   sincospi(-2.0 * (double)(r * k) / (double)(1 << (d.lgLs[b] + d.lgR[b])), &sn, &cs);
   dst[t] = make_float2((float)cs, (float)sn);
@@ -458,9 +458,9 @@ __global__ void small_tab_admm_k(const double2* __restrict__ chat, int64_t n, fl
   abs2[k] = a.x * a.x + a.y * a.y;
 }
 
-template <int LG>
+template <int LG, bool FULL>
 constexpr size_t small_smem(bool dense) {
-  return sizeof(float2) * (2 * small_buf<LG>() + ((SmallShape<LG>::kTw + 1) & ~1)) +
+  return sizeof(float2) * (2 * small_buf<LG>() + ((SmallTw<LG, FULL>::kTw + 1) & ~1)) +
          (dense ? sizeof(float2) << LG : 0);
 }
 
@@ -469,13 +469,13 @@ cudaError_t opt_in_smem(const void* fn, size_t smem) {
                           : cudaSuccess;
 }
 
-// LG = 13 (64 values of padding per 1024 and 62 KiB of twiddles: 201 KiB)
+// LG = 13 (64 values of padding per 1024 and 84 KiB of twiddles: 220 KiB)
 // fits without a dense y, so only ADMM takes it.
 template <int LG>
 cudaError_t class_run(bool admm, const SmallInst* inst, int count, const SmallScalars* sc, const float* y, float* xz,
                       int iters, cudaStream_t s) {
   const void* fn = nullptr;
-  size_t smem = small_smem<LG>(!admm);
+  size_t smem = small_smem<LG, true>(!admm);
   if (admm) fn = (const void*)class_admm_k<LG>;
   else if constexpr (LG <= SMALL_LG_MAX) fn = (const void*)class_ista_k<LG>;
   if (!fn) return cudaErrorInvalidValue;
@@ -491,11 +491,11 @@ cudaError_t small_run(SmallKind kind, const SmallArgs& a, cudaStream_t s) {
   const void* fn = nullptr;
   size_t smem = 0;
   switch (kind) {
-    case SMALL_ISTA: fn = (const void*)small_ista_k<LG>; smem = small_smem<LG>(true); break;
-    case SMALL_ADMM: fn = (const void*)small_admm_k<LG>; smem = small_smem<LG>(false); break;
-    case SMALL_POWER: fn = (const void*)small_power_k<LG>; smem = small_smem<LG>(false); break;
-    case SMALL_FWD: fn = (const void*)small_product_k<LG, true>; smem = small_smem<LG>(true); break;
-    case SMALL_ADJ: fn = (const void*)small_product_k<LG, false>; smem = small_smem<LG>(true); break;
+    case SMALL_ISTA: fn = (const void*)small_ista_k<LG>; smem = small_smem<LG, false>(true); break;
+    case SMALL_ADMM: fn = (const void*)small_admm_k<LG>; smem = small_smem<LG, false>(false); break;
+    case SMALL_POWER: fn = (const void*)small_power_k<LG>; smem = small_smem<LG, false>(false); break;
+    case SMALL_FWD: fn = (const void*)small_product_k<LG, true>; smem = small_smem<LG, false>(true); break;
+    case SMALL_ADJ: fn = (const void*)small_product_k<LG, false>; smem = small_smem<LG, false>(true); break;
   }
   const cudaError_t e = opt_in_smem(fn, smem);
   if (e != cudaSuccess) return e;
@@ -527,20 +527,20 @@ cudaError_t launch_small_class(bool admm, int lgN, const SmallInst* inst, int co
   return cudaErrorInvalidValue;
 }
 
-static SmallTwStages tw_stages(int lgN) {
+static SmallTwStages tw_stages(int lgN, bool full) {
   switch (lgN) {
-    case 13: return small_tw_stages<13>();
-#define CS_X(L) case L: return small_tw_stages<L>();
+    case 13: return small_tw_stages<13, true>();   // size classes only
+#define CS_X(L) case L: return full ? small_tw_stages<L, true>() : small_tw_stages<L, false>();
     CS_SMALL_LG(CS_X)
 #undef CS_X
   }
   return SmallTwStages{};
 }
 
-int small_tw_count(int lgN) { return tw_stages(lgN).total; }
+int small_tw_count(int lgN, bool full) { return tw_stages(lgN, full).total; }
 
-cudaError_t launch_small_tw(int lgN, float2* tw, cudaStream_t s) {
-  const SmallTwStages d = tw_stages(lgN);
+cudaError_t launch_small_tw(int lgN, bool full, float2* tw, cudaStream_t s) {
+  const SmallTwStages d = tw_stages(lgN, full);
   small_tw_k<<<(unsigned)((d.total + 255) / 256), 256, 0, s>>>(tw, d);
   return cudaGetLastError();
 }

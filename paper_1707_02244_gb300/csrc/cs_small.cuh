@@ -36,39 +36,68 @@ template <int LG> struct SmallShape {
   static constexpr int kLgM1 = kLgM > kLgE ? (kLgM + 1) / 2 : kLgM;
   static constexpr int kLgM2 = kLgM - kLgM1;
   static_assert(kLgM >= 0 && kLgM1 <= kLgE && kLgM2 <= kLgE, "radices");
-  // twiddle blocks: forward middle 1, middle 2, last; inverse middle 2, middle 1, last (radix R1)
-  static constexpr int kF1 = 0;
-  static constexpr int kF2 = kF1 + (kLgM1 ? tw_rows(kLgM1) << kLg1 : 0);
-  static constexpr int kFL = kF2 + (kLgM2 ? tw_rows(kLgM2) << (kLg1 + kLgM1) : 0);
-  static constexpr int kI2 = kFL + (tw_rows(kLgL) << (LG - kLgL));
-  static constexpr int kI1 = kI2 + (kLgM2 ? tw_rows(kLgM2) << kLgL : 0);
-  static constexpr int kIL = kI1 + (kLgM1 ? tw_rows(kLgM1) << (kLgL + kLgM2) : 0);
-  static constexpr int kTw = kIL + (tw_rows(kLg1) << (LG - kLg1));
 };
 
-// The same description for the host and the table kernel: stage b holds
-// rows r(row) of w_{Ls R}^(r k) at off + row Ls + k.
+// Twiddle blocks: forward middle 1, middle 2, last; inverse middle 2, middle
+// 1, last (radix R1 = 2 RL).
+//
+// FULL: every twiddle is a table value rounded once.  The two last stages take
+// the same roots w_N^(r k), so the inverse one reads the forward one's rows:
+// r < RL directly, an even r >= RL as row r / 2 at 2k; its own block holds the
+// odd r > RL only (8192-long transforms fit the CTA's shared memory this way).
+// Otherwise the higher powers are products of two table values (see
+// stage_twiddle).
+//
+// The batch's size classes take FULL: the solver they replaced did too, and
+// with products their ADMM error against 64 bits was 10 to 15 %
+// larger (20 iterations, n = 1024 .. 8192; within 2 % with FULL, at the same time: a batch
+// fills the chip, 8.50 against 8.53 ms for 256 instances).  One instance of a
+// plan takes products: bound by one SM's shared-memory pipe, it is 10 % slower
+// with FULL (500 ISTA iterations at n = 4096: 2.04 against 2.25 ms), and either
+// way it rounds less than the four-step passes it replaced (n = 1024 .. 4096:
+// products 0.79 .. 0.84 of a product's error, ISTA 0.95, ADMM 0.9; FULL 0.75 ..
+// 0.80, 0.94, 0.8).
+template <int LG, bool FULL> struct SmallTw {
+  using S = SmallShape<LG>;
+  static constexpr int kF1 = 0;
+  static constexpr int kF2 = kF1 + (S::kLgM1 ? tw_rows(S::kLgM1, FULL) << S::kLg1 : 0);
+  static constexpr int kFL = kF2 + (S::kLgM2 ? tw_rows(S::kLgM2, FULL) << (S::kLg1 + S::kLgM1) : 0);
+  static constexpr int kI2 = kFL + (tw_rows(S::kLgL, FULL) << (LG - S::kLgL));
+  static constexpr int kI1 = kI2 + (S::kLgM2 ? tw_rows(S::kLgM2, FULL) << S::kLgL : 0);
+  static constexpr int kIL = kI1 + (S::kLgM1 ? tw_rows(S::kLgM1, FULL) << (S::kLgL + S::kLgM2) : 0);
+  static constexpr int kTw = kIL + ((FULL ? S::E / 4 : tw_rows(S::kLg1, false)) << (LG - S::kLg1));
+};
+
+// The same description for the host and the table kernel: row `row` of stage b
+// holds w_{Ls R}^(r k) at off + row Ls + k, r = small_tw_r(stages, b, row).
 struct SmallTwStages {
   int count;
   int off[6], lgLs[6], lgR[6];
   int total;
+  bool full;
 };
-template <int LG> SmallTwStages small_tw_stages() {
+__host__ __device__ inline int small_tw_r(const SmallTwStages& d, int b, int row) {
+  if (d.full && b + 1 == d.count) return (1 << (d.lgR[b] - 1)) + 1 + 2 * row;   // last inverse stage: odd r > RL
+  return tw_row_r(d.lgR[b], row, d.full);
+}
+template <int LG, bool FULL> SmallTwStages small_tw_stages() {
   using S = SmallShape<LG>;
+  using T = SmallTw<LG, FULL>;
   SmallTwStages d{};
+  d.full = FULL;
   auto add = [&](int off, int lgLs, int lgR) {
     if (lgR == 0) return;
     d.off[d.count] = off;
     d.lgLs[d.count] = lgLs;
     d.lgR[d.count++] = lgR;
   };
-  add(S::kF1, S::kLg1, S::kLgM1);
-  add(S::kF2, S::kLg1 + S::kLgM1, S::kLgM2);
-  add(S::kFL, LG - S::kLgL, S::kLgL);
-  add(S::kI2, S::kLgL, S::kLgM2);
-  add(S::kI1, S::kLgL + S::kLgM2, S::kLgM1);
-  add(S::kIL, LG - S::kLg1, S::kLg1);
-  d.total = S::kTw;
+  add(T::kF1, S::kLg1, S::kLgM1);
+  add(T::kF2, S::kLg1 + S::kLgM1, S::kLgM2);
+  add(T::kFL, LG - S::kLgL, S::kLgL);
+  add(T::kI2, S::kLgL, S::kLgM2);
+  add(T::kI1, S::kLgL + S::kLgM2, S::kLgM1);
+  add(T::kIL, LG - S::kLg1, S::kLg1);
+  d.total = T::kTw;
   return d;
 }
 
@@ -79,7 +108,7 @@ __host__ __device__ constexpr int padP(int i) { return i + (i >> 4); }
 template <int LG> __host__ __device__ constexpr int small_buf() { return padP(1 << LG); }   // float2 per exchange buffer
 
 // One middle stage (span 2^LGLS, radix 2^LGR) from buffer a to buffer b.
-template <int LG, int LGLS, int LGR, int DIR>
+template <int LG, bool FULL, int LGLS, int LGR, int DIR>
 __device__ __forceinline__ void small_mid(const float2* a, float2* b, const float2* tw) {
   using S = SmallShape<LG>;
   constexpr int R = 1 << LGR, LS = 1 << LGLS, B = S::E / R, ST = S::N / R;
@@ -94,7 +123,7 @@ __device__ __forceinline__ void small_mid(const float2* a, float2* b, const floa
 #pragma unroll
     for (int i = 0; i < B; ++i) {
       const int j = threadIdx.x + i * S::NA, k = j & (LS - 1);
-      stage_twiddle<R, DIR>(v[i], tw, LS, k);
+      stage_twiddle<R, DIR, FULL>(v[i], tw, LS, k);
       dft<R, DIR>(v[i]);
       float2* q = b + padP(((j - k) << LGR) + k);
 #pragma unroll
@@ -104,16 +133,36 @@ __device__ __forceinline__ void small_mid(const float2* a, float2* b, const floa
   __syncthreads();
 }
 
+// Twiddles of the last inverse stage, butterfly k.
+template <int LG, bool FULL>
+__device__ __forceinline__ void small_twiddle_last(float2* v, const float2* tw, int k) {
+  using S = SmallShape<LG>;
+  using T = SmallTw<LG, FULL>;
+  constexpr int R1 = S::E, RL = S::E / 2, M = S::N / RL, ST1 = S::N / R1;
+  if constexpr (FULL) {
+#pragma unroll
+    for (int r = 1; r < R1; ++r) {
+      const float2 w = r < RL        ? tw[T::kFL + (r - 1) * M + k]
+                       : (r & 1) == 0 ? tw[T::kFL + (r / 2 - 1) * M + 2 * k]
+                                      : tw[T::kIL + (r - RL) / 2 * ST1 + k];
+      v[r] = cmulc(v[r], w);
+    }
+  } else {
+    stage_twiddle<R1, +1, false>(v, tw + T::kIL, ST1, k);
+  }
+}
+
 // v (element tid + r N/R1 in v[r]) -> inverse FFT of op(forward FFT of v),
 // unnormalised, in the same order.  op(k, za, zb) is applied to every pair
 // (k, N - k), k <= N/2; for the self-pairs k = 0 and N/2 za and zb hold the
 // same value and za is kept.  S0, S1: exchange buffers; on return S0 and S1
 // may still be read by other threads of the CTA only in the way the next call
 // allows (it writes S0 first, whose last reader is behind a barrier).
-template <int LG, class OP>
+template <int LG, bool FULL, class OP>
 __device__ __forceinline__ void small_conv(float2 (&v)[SmallShape<LG>::E], float2* S0, float2* S1,
                                            const float2* tw, const OP& op) {
   using S = SmallShape<LG>;
+  using T = SmallTw<LG, FULL>;
   constexpr int N = S::N, R1 = S::E, RL = S::E / 2, M = N / RL, ST1 = N / R1;
   const int tid = threadIdx.x;
   const bool act = tid < S::NA;
@@ -126,11 +175,11 @@ __device__ __forceinline__ void small_conv(float2 (&v)[SmallShape<LG>::E], float
   }
   __syncthreads();
   if constexpr (S::kLgM1 > 0) {
-    small_mid<LG, S::kLg1, S::kLgM1, -1>(a, b, tw + S::kF1);
+    small_mid<LG, FULL, S::kLg1, S::kLgM1, -1>(a, b, tw + T::kF1);
     float2* t = a; a = b; b = t;
   }
   if constexpr (S::kLgM2 > 0) {
-    small_mid<LG, S::kLg1 + S::kLgM1, S::kLgM2, -1>(a, b, tw + S::kF2);
+    small_mid<LG, FULL, S::kLg1 + S::kLgM1, S::kLgM2, -1>(a, b, tw + T::kF2);
     float2* t = a; a = b; b = t;
   }
   if (act) {
@@ -142,8 +191,8 @@ __device__ __forceinline__ void small_conv(float2 (&v)[SmallShape<LG>::E], float
       x[r] = q0[padP(r * M)];
       y[r] = q1[padP(r * M)];
     }
-    stage_twiddle<RL, -1>(x, tw + S::kFL, M, j0);
-    stage_twiddle<RL, -1>(y, tw + S::kFL, M, j1);
+    stage_twiddle<RL, -1, FULL>(x, tw + T::kFL, M, j0);
+    stage_twiddle<RL, -1, FULL>(y, tw + T::kFL, M, j1);
     dft<RL, -1>(x);
     dft<RL, -1>(y);
     float2 p[RL], w[RL];   // frequency order
@@ -187,11 +236,11 @@ __device__ __forceinline__ void small_conv(float2 (&v)[SmallShape<LG>::E], float
   __syncthreads();
   { float2* t = a; a = b; b = t; }
   if constexpr (S::kLgM2 > 0) {
-    small_mid<LG, S::kLgL, S::kLgM2, +1>(a, b, tw + S::kI2);
+    small_mid<LG, FULL, S::kLgL, S::kLgM2, +1>(a, b, tw + T::kI2);
     float2* t = a; a = b; b = t;
   }
   if constexpr (S::kLgM1 > 0) {
-    small_mid<LG, S::kLgL + S::kLgM2, S::kLgM1, +1>(a, b, tw + S::kI1);
+    small_mid<LG, FULL, S::kLgL + S::kLgM2, S::kLgM1, +1>(a, b, tw + T::kI1);
     float2* t = a; a = b; b = t;
   }
   if (act) {
@@ -199,7 +248,7 @@ __device__ __forceinline__ void small_conv(float2 (&v)[SmallShape<LG>::E], float
     float2 u[R1];
 #pragma unroll
     for (int r = 0; r < R1; ++r) u[r] = q[padP(r * ST1)];
-    stage_twiddle<R1, +1>(u, tw + S::kIL, ST1, tid);
+    small_twiddle_last<LG, FULL>(u, tw, tid);
     dft<R1, +1>(u);
 #pragma unroll
     for (int r = 0; r < R1; ++r) v[r] = u[out_slot<R1>(r)];
