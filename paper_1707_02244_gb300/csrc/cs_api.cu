@@ -386,26 +386,30 @@ cudaError_t run_chunk(cs_plan_s* p, SolveKind kind, int len, bool final_chunk, b
   return cudaGraphLaunch(it->second, p->stream);
 }
 
-// Iterate in chunks of check_every; with a monitor tolerance, stop at the
-// first check point whose NMSE meets it.
+// Iterate up to the check points, every check_every iterations; with a monitor
+// tolerance, stop at the first one whose NMSE meets it.
 // step(done, len, final chunk, statistics) enqueues iterations done .. done +
-// len - 1; at most `most` in one chunk when nobody watches.
+// len - 1.  `most` > 0: the solver takes any number of iterations in one
+// launch, so a chunk ends at a check point that is watched and otherwise at
+// `most` iterations, whatever check_every is.
 template <class F>
 cudaError_t solve_loop(cs_plan_s* p, int iters, int* iters_run, int* converged, bool need_stats, int most, F&& step) {
   *iters_run = 0;
   *converged = 0;
   const bool watch = p->xtrue != nullptr && p->tol > 0.0;
-  const int ce = watch || most < p->check_every ? p->check_every : most;
+  const int ce = p->check_every;
   int done = 0;
   while (done < iters) {
-    const int len = (iters - done) < ce ? (iters - done) : ce;
-    const bool final_chunk = done + len == iters;
+    int len = iters - done;
+    if ((watch || most == 0) && len > ce - done % ce) len = ce - done % ce;
+    if (most > 0 && len > most) len = most;
+    const bool final_chunk = done + len == iters, check = watch && (done + len) % ce == 0;
     // the statistics of a check point are formed where somebody reads them:
     // by the monitor at every one, else by the caller's record at the last
-    cudaError_t e = step(done, len, final_chunk, watch || (final_chunk && need_stats));
+    cudaError_t e = step(done, len, final_chunk, check || (final_chunk && (need_stats || watch)));
     if (e != cudaSuccess) return e;
     done += len;
-    if (watch && !final_chunk) {
+    if (check && !final_chunk) {
       e = read_back(p);
       if (e != cudaSuccess) return e;
       const double nm = p->host_stats[ST_ERR2] / p->xtrue2;
@@ -444,7 +448,8 @@ void fill_stats(const cs_plan_s* p, cs_stats* st, int iters_run, int converged, 
   (void)admm;
 }
 
-// Longest single-CTA launch (iterations): tens of milliseconds.
+// Longest launch of a single-CTA or cluster solve, in iterations: 20 to 110 ms
+// (2 to 11 us an iteration).
 constexpr int SMALL_CHUNK = 10000;
 
 SmallArgs small_args(const cs_plan_s* p, bool admm) {

@@ -1,0 +1,62 @@
+"""How a solve is cut into launches: the longest launch, check points, state
+that is carried from one chunk to the next, and the record at a check point,
+on each of the three solvers (one CTA, one cluster of CTAs, the passes).
+
+Tolerances: 1e-5 against the FP64 oracle as in test_gpu_shapes.py (a few
+iterations from zero); bit equality where the same kernel does the same
+iterations in another number of launches.
+"""
+import numpy as np
+import pytest
+
+import oracle.cs_oracle as O
+import synth
+from gpu_util import f32, host, rel_l2, to_dev, torch_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def cs():
+    import paper_1707_02244_gb300 as cs
+    return cs
+
+
+def _plan(cs, n, seed):
+    torch, dev = torch_dev()
+    m = n // 3 | 1
+    g = synth.rng(seed)
+    c = synth.gaussian_c(g, n, m)
+    rows = synth.draw_rows(g, n, m)
+    x = synth.k_sparse(g, n, max(2, n // 100))
+    chat = O.spectrum(c)
+    y = (O.forward_fft(chat, rows, x) + 1e-3 * g.standard_normal(m)).astype(np.float32)
+    plan = cs.cs_plan(n, m, rows, c, torch.cuda.current_stream(dev))
+    return plan, c, rows, x, y, f32(0.9 / np.max(np.abs(chat) ** 2))
+
+
+@pytest.mark.parametrize("n", [64, 1 << 13])
+def test_launch_length_is_bounded(cs, n):
+    """No launch runs more than 10000 iterations, whatever check_every is."""
+    torch, dev = torch_dev()
+    plan, _, _, x_true, y, tau = _plan(cs, n, 8100 + n)
+    yd, xt = to_dev(y), to_dev(x_true)
+    try:
+        ref, x = torch.zeros(n, device=dev), torch.zeros(n, device=dev)
+        assert cs.cs_ista(plan, yd, 1e-3, tau, 25000, ref)["launches"] == 3
+        zref, z = torch.empty(n, device=dev), torch.empty(n, device=dev)
+        count = cs.cs_admm(plan, yd, 1e-3, 1.0, 25000, zref)["launches"]
+        cs.cs_set_monitor(plan, None, 0.0, 10 ** 9)
+        assert cs.cs_ista(plan, yd, 1e-3, tau, 25000, x)["launches"] == 3
+        assert torch.equal(x, ref)
+        assert cs.cs_admm(plan, yd, 1e-3, 1.0, 25000, z)["launches"] == count
+        assert torch.equal(z, zref)
+        # watched, with a tolerance that is never met: launches end at 10000,
+        # 15000, 25000 (the check points are 15000 apart)
+        cs.cs_set_monitor(plan, xt, 1e-30, 15000)
+        x.zero_()
+        st = cs.cs_ista(plan, yd, 1e-3, tau, 25000, x)
+        assert st["launches"] == 3 and st["iters_run"] == 25000 and st["converged"] == 0
+        assert torch.equal(x, ref)
+    finally:
+        plan.close()
