@@ -187,10 +187,12 @@ cs_status cs_plan_2d(cs_plan_t* out, int64_t n0, int64_t n1, int64_t m, const in
  * tau is held fixed (it is not differentiated through ||A||^2).  The
  * soft threshold's derivative is taken as 1 where |u| > tau lambda and 0
  * elsewhere (its value at the kink is a convention).
- * The forward iterates are kept every K steps (checkpoints, (T/K + 1) n
+ * The forward iterates are kept every K steps (checkpoints, ceil(T/K) n
  * floats) and each segment of K steps is replayed before it is
- * back-propagated ((2K + 4) n more floats, allocated by the first call and
- * kept by the plan).  1 <= K <= T.  Asynchronous; errors as cs_ista.
+ * back-propagated ((3K + 4) n + m more floats, allocated by the first call
+ * and kept by the plan).  Where that does not fit the device, the plan takes segments of about sqrt(T / 3) steps instead, which
+ * need the least memory and give the same result; CS_ERR_NOMEM if those do
+ * not fit either.  1 <= K <= T.  Asynchronous; errors as cs_ista.
  * Uses the plan's solver state: not concurrent with cs_ista / cs_admm. */
 cs_status cs_grad(cs_plan_t plan, const float* y, float lambda, float tau, int T, int K,
                   const float* gx_T, float* dc, float* dlambda, float* dy);

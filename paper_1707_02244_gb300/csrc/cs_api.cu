@@ -2,6 +2,7 @@
 // argument checks, CUDA-graph capture of the iteration loop, monitoring.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -77,6 +78,7 @@ struct cs_plan_s {
   // unrolled-ISTA gradient (cs_grad): allocated at the first call, grown on demand
   struct Grad {
     int ck_cap = 0, seg_cap = 0;
+    bool tight = false;      // the segments asked for did not fit: short ones (see cs_grad)
     float* ckpt = nullptr;   // [ck_cap][n]  x(sK), tile order
     float* seg = nullptr;    // [seg_cap + 1][n]  x(t) of the segment being replayed
     float2* rw = nullptr;    // [seg_cap][n/2]  column transform of r(t)
@@ -1128,10 +1130,13 @@ cudaError_t grad_reserve(cs_plan_s* p, int ck, int seg) {
     }
   }
   const int nck = ck > G.ck_cap ? ck : G.ck_cap, nseg = seg > G.seg_cap ? seg : G.seg_cap;
-  void* old[] = {G.ckpt, G.seg, G.rw, G.xw, G.g, G.w, G.dy, G.gacc, G.gpart, G.ca};
-  for (void* b : old)
-    if (b) cudaFree(b);
-  G = cs_plan_s::Grad{};
+  auto drop = [&] {
+    void* old[] = {G.ckpt, G.seg, G.rw, G.xw, G.g, G.w, G.dy, G.gacc, G.gpart, G.ca};
+    for (void* b : old)
+      if (b) cudaFree(b);
+    G = cs_plan_s::Grad{};
+  };
+  drop();
   const size_t n = (size_t)p->n;
   e = dalloc(&G.ckpt, (size_t)nck * n);
   if (e == cudaSuccess) e = dalloc(&G.seg, (size_t)(nseg + 1) * n);
@@ -1146,6 +1151,9 @@ cudaError_t grad_reserve(cs_plan_s* p, int ck, int seg) {
   if (e == cudaSuccess) {
     G.ck_cap = nck;
     G.seg_cap = nseg;
+  } else {
+    drop();
+    cudaGetLastError();   // reported here, not by the next launch
   }
   return e;
 }
@@ -1228,9 +1236,24 @@ cs_status cs_grad(cs_plan_t p, const float* y, float lambda, float tau, int T, i
     return CS_ERR_ARG;
   if (p->gi.twod) return CS_ERR_UNSUPPORTED;
   cudaStream_t s = p->stream;
-  const int S = (T + K - 1) / K;   // segments; segment s covers steps [sK, min((s+1)K, T))
-  CS_TRY(grad_reserve(p, S, K));
   auto& G = p->gr;
+  // S segments; segment s covers steps [sK, min((s+1)K, T)).  They take S + 3K
+  // vectors of n.  Where those do not fit, segments of about sqrt(T/3) steps
+  // take the fewest: each step is replayed once whatever K is, so the results
+  // are the same bits and the time is too.
+  const int Kmin = std::max(1, std::min(K, (int)std::lround(std::sqrt(T / 3.0))));
+  bool tight = G.tight;
+  if (tight) K = Kmin;
+  int S = (T + K - 1) / K;
+  cudaError_t er = grad_reserve(p, S, K);
+  if (er == cudaErrorMemoryAllocation && K > Kmin) {
+    tight = true;
+    K = Kmin;
+    S = (T + K - 1) / K;
+    er = grad_reserve(p, S, K);
+  }
+  CS_TRY(er);
+  G.tight = tight;
   const size_t n = (size_t)p->n;
   p->launches = 0;
   const float thr = (float)((double)tau * (double)lambda);

@@ -35,6 +35,30 @@ def _plan(cs, n, seed):
     return plan, c, rows, x, y, f32(0.9 / np.max(np.abs(chat) ** 2))
 
 
+def test_grad_segments_that_do_not_fit(cs):
+    """K = T = 8000 at n = 2^22: 24000 vectors, 375 GiB.  The plan takes shorter
+    segments, which give the same gradient."""
+    torch, dev = torch_dev()
+    n, T = 1 << 22, 8000
+    plan, _, _, _, y, tau = _plan(cs, n, 8190)
+    g = torch.Generator(device=dev)
+    g.manual_seed(3)
+    gx = torch.randn(n, generator=g, device=dev)
+    torch.cuda.empty_cache()
+    out = []
+    try:
+        for K in (T, 100, T):
+            dc, dl, dy = (torch.empty(k, device=dev) for k in (n, 1, plan.m))
+            cs.cs_grad(plan, to_dev(y), 0.05, tau, T, K, gx, dc, dl, dy)
+            out.append((dc, dl, dy))
+        assert cs.cs_status_sync(plan) == 0
+    finally:
+        plan.close()
+    for got in (out[0], out[2]):
+        assert all(torch.equal(a, b) for a, b in zip(got, out[1]))
+    assert float(out[1][0].norm()) > 0.0
+
+
 @pytest.mark.parametrize("n", [64, 1 << 13])
 def test_launch_length_is_bounded(cs, n):
     """No launch runs more than 10000 iterations, whatever check_every is."""
