@@ -156,8 +156,11 @@ cs_status cs_admm_ex(cs_plan_t plan, const float* y, float lambda,
  *   0 mid pass C x      1 column pass residual   2 mid pass C^T r
  *   3 column pass ISTA update                   4 mid pass ADMM x-update
  *   5 column pass ADMM updates
- * For timing with CUDA events around the call.  Errors: CS_ERR_ARG
- * (pass_id, reps < 1, no earlier solve of that kind). */
+ * For timing with CUDA events around the call.  A solve that runs in one
+ * launch (1D, n <= 2^15) has no passes: the hook then times the pass kernels
+ * of that length, and its first call after such a solve also lays out their
+ * inputs from the buffers that the solve named.  Errors: CS_ERR_ARG (pass_id, reps < 1, no
+ * earlier solve of that kind). */
 cs_status cs_profile_pass(cs_plan_t plan, int pass_id, int reps);
 
 /* Plan of the 2D operator (Sec. 7, compressed deblurring): A = P H with H

@@ -73,8 +73,14 @@ struct cs_plan_s {
   } sml;
   bool cluster_i = false, cluster_a = false;   // one cluster solves the instance
   float2 *twn_i = nullptr, *twn_a = nullptr;   // its four-step twiddles, exp(-2 pi i q / N)
-  CallArgs last_ca{};              // arguments of the last single-CTA solve: cs_profile_pass sends them first
-  bool ca_stale = false;
+  // The last solve ran in one launch and left the passes' inputs alone:
+  // cs_profile_pass lays them out from these first.
+  struct OneLaunch {
+    bool pending = false;
+    CallArgs a{};
+    const float* y = nullptr;
+    const float* state[4] = {};    // ADMM: v, z, mu, nu in natural order, or null (zero)
+  } one;
   // unrolled-ISTA gradient (cs_grad): allocated at the first call, grown on demand
   struct Grad {
     int ck_cap = 0, seg_cap = 0;
@@ -879,8 +885,7 @@ cs_status cs_ista(cs_plan_t p, const float* y, float lambda, float tau, int iter
     sa.x = x;
     sa.thr = a.thr;
     sa.tau = tau;
-    p->last_ca = a;
-    p->ca_stale = true;
+    p->one = {true, a, y, {}};
     CS_TRY(solve_loop(p, iters, &run, &conv, stats != nullptr, SMALL_CHUNK,
                       [&](int, int len, bool, bool st) {
                         sa.iters = len;
@@ -895,8 +900,7 @@ cs_status cs_ista(cs_plan_t p, const float* y, float lambda, float tau, int iter
     ca.x = x;
     ca.thr = a.thr;
     ca.tau = tau;
-    p->last_ca = a;
-    p->ca_stale = true;
+    p->one = {true, a, y, {}};
     CS_TRY(solve_loop(p, iters, &run, &conv, stats != nullptr, SMALL_CHUNK,
                       [&](int, int len, bool, bool st) {
                         ca.iters = len;
@@ -906,7 +910,7 @@ cs_status cs_ista(cs_plan_t p, const float* y, float lambda, float tau, int iter
                         return e == cudaSuccess && st ? launch_finalize(p->partials, cluster_ctas(), p->stats, s) : e;
                       }));
   } else {
-    p->ca_stale = false;
+    p->one.pending = false;
     CS_TRY(launch_set_args(a, p->ca, s));
     CS_TRY(launch_scatter_y(y, p->si.pos, p->m, p->si.ys, p->status, s));
     p->launches += 2;
@@ -979,8 +983,7 @@ cs_status admm_impl(cs_plan_t p, const float* y, float lambda, const cs_admm_par
   p->ista_args = false;
   int run = 0, conv = 0;
   if (small) {
-    p->last_ca = a;
-    p->ca_stale = true;
+    p->one = {true, a, y, {v, z, mu, nu}};
     SmallArgs sa{};
     ClusterArgs ca{};
     auto fill = [&](auto& q) {
@@ -1029,7 +1032,7 @@ cs_status admm_impl(cs_plan_t p, const float* y, float lambda, const cs_admm_par
       return launch_finalize(p->partials, cluster_ctas(), p->stats, s);
     }));
   } else {
-    p->ca_stale = false;
+    p->one.pending = false;
     CS_TRY(launch_set_args(a, p->ca, s));
     CS_TRY(launch_scatter_y(y, p->sa.pos, p->m, p->sa.ys, p->status, s));
     p->launches += 2;
@@ -1083,9 +1086,23 @@ cs_status cs_profile_pass(cs_plan_t p, int pass_id, int reps) {
   if (pass_id <= 3 && !p->ista_args) return CS_ERR_ARG;
   if (pass_id >= 4 && !p->admm_args) return CS_ERR_ARG;
   cudaStream_t s = p->stream;
-  if (p->ca_stale) {
-    CS_TRY(launch_set_args(p->last_ca, p->ca, s));
-    p->ca_stale = false;
+  if (p->one.pending) {
+    const auto& o = p->one;
+    CS_TRY(launch_set_args(o.a, p->ca, s));
+    if (p->ista_args) {
+      CS_TRY(launch_scatter_y(o.y, p->si.pos, p->m, p->si.ys, p->status, s));
+      CS_TRY(launch_to_tile(o.a.src, p->xi_t, p->gi, 1, s));
+      CS_TRY(launch_col(COL_LOAD, kparams(p, p->gi, 0), s));
+    } else {
+      CS_TRY(launch_scatter_y(o.y, p->sa.pos, p->m, p->sa.ys, p->status, s));
+      float* tiled[4] = {p->av, p->az, p->amu, p->anu};
+      for (int i = 0; i < 4; ++i) {
+        if (o.state[i]) CS_TRY(launch_to_tile(o.state[i], tiled[i], p->ga, 0, s));
+        else CS_TRY(cudaMemsetAsync(tiled[i], 0, p->n * sizeof(float), s));
+      }
+      CS_TRY(launch_col(COL_ADMM_INIT, kparams(p, p->ga, 0), s));
+    }
+    p->one.pending = false;
   }
   for (int r = 0; r < reps; ++r) {
     switch (pass_id) {

@@ -35,6 +35,34 @@ def _plan(cs, n, seed):
     return plan, c, rows, x, y, f32(0.9 / np.max(np.abs(chat) ** 2))
 
 
+@pytest.mark.parametrize("n", [64, 4096, 1 << 13, 1 << 15, 1 << 17])
+def test_profile_pass_inputs(cs, n):
+    """The pass kernels that the measurement hook launches find inputs laid out:
+    by the solve on the pass path, else by the hook from the buffers that the
+    solve named (so that it sees, and reports, what y holds by then)."""
+    torch, dev = torch_dev()
+    plan, _, _, _, y, tau = _plan(cs, n, 8200 + n)
+    yd = to_dev(y)
+    x, z = torch.zeros(n, device=dev), torch.empty(n, device=dev)
+    try:
+        for solve, out, passes, one_launch in (
+                (lambda o: cs.cs_ista(plan, yd, 1e-3, tau, 3, o, stats=False), x, (0, 1, 2, 3), n <= 1 << 15),
+                (lambda o: cs.cs_admm(plan, yd, 1e-3, 1.0, 3, o, stats=False), z, (4, 5), n <= 1 << 15)):
+            out.zero_()
+            solve(out)
+            want = out.clone()
+            yd[0] = float("inf")
+            for k in passes:
+                cs.cs_profile_pass(plan, k, 2)
+            assert cs.cs_status_sync(plan) == (5 if one_launch else 0)   # CS_ERR_NONFINITE
+            yd.copy_(torch.from_numpy(y))
+            out.zero_()
+            solve(out)
+            assert torch.equal(out, want) and cs.cs_status_sync(plan) == 0
+    finally:
+        plan.close()
+
+
 def test_grad_segments_that_do_not_fit(cs):
     """K = T = 8000 at n = 2^22: 24000 vectors, 375 GiB.  The plan takes shorter
     segments, which give the same gradient."""
