@@ -52,6 +52,7 @@ import hashlib
 import json
 import os
 import pathlib
+import re
 import statistics
 import subprocess
 import sys
@@ -279,13 +280,26 @@ def pass_bytes(pid, n, m):
     return 16 * n + 16 * n + 4 * m + n // 4   # ADMM column pass: W, mu, nu in/out, y, mask
 
 
-PASS_SOURCES = ("cs_col.cu", "cs_mid.cu", "cs_passes.cuh", "cs_fft.cuh", "cs_internal.h")
+PASS_UNITS = ("cs_col.cu", "cs_mid.cu")   # the units that instantiate the pass kernels of n = 2^22
+
+
+def pass_sources():
+    """The pass kernels' units and every file of csrc that they include."""
+    src, todo = set(), list(PASS_UNITS)
+    while todo:
+        name = todo.pop()
+        f = ROOT / "paper_1707_02244_gb300" / "csrc" / name
+        if name in src or not f.exists():
+            continue
+        src.add(name)
+        todo += re.findall(r'^\s*#include "([\w.]+)"', f.read_text(), flags=re.M)
+    return sorted(src)
 
 
 def pass_sources_digest():
     """sha256[:16] of the sources that define the pass kernels."""
     src = hashlib.sha256()
-    for name in PASS_SOURCES:
+    for name in pass_sources():
         src.update((ROOT / "paper_1707_02244_gb300" / "csrc" / name).read_bytes())
     return src.hexdigest()[:16]
 
