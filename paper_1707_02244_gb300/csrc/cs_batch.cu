@@ -313,9 +313,9 @@ cs_status cs_batch_plan(cs_batch_t* out, int count, const int64_t* n, const int6
   std::stable_sort(b->large.begin(), b->large.end(), [&](int a, int c2) { return n[a] > n[c2]; });
   // The size-class launches of the small instances go to the side streams
   // longest first, each to the stream with the least work so far (cost ~ n
-  // per iteration; a class runs its instances side by side, about 2 * 152 at
-  // a time); the grouped launches of the large instances run on the batch's
-  // stream.
+  // per iteration and wave; a wave is what the chip holds of the class's ADMM
+  // CTAs, one per SM at n = 8192 and more below); the grouped launches of the
+  // large instances run on the batch's stream.
   for (size_t j = 0; j < b->small.size();) {
     const int lg = hd[b->small[j]].lgn;
     size_t e = j;
@@ -328,7 +328,13 @@ cs_status cs_batch_plan(cs_batch_t* out, int count, const int64_t* n, const int6
     std::vector<Item> items;
     for (size_t j = 0; j < b->classes.size(); ++j) {
       const auto& cl = b->classes[j];
-      items.push_back({(double)(int64_t(1) << cl.lgn) * (double)((cl.count + 303) / 304), 0, (int)j});
+      int wave = 0;
+      const cudaError_t e = small_class_wave(cl.lgn, &wave);
+      if (e != cudaSuccess) {
+        batch_free(b);
+        return cstat(e);
+      }
+      items.push_back({(double)(int64_t(1) << cl.lgn) * (double)((cl.count + wave - 1) / wave), 0, (int)j});
     }
     std::stable_sort(items.begin(), items.end(), [](const Item& a, const Item& c2) { return a.cost > c2.cost; });
     double load[NSIDE_MAX] = {};

@@ -243,6 +243,8 @@ struct SmallInst {
 struct SmallScalars {      // per call and instance
   float thr, tau, rho, sigma, tau1, tau2, d_on, d_off;
 };
+// Instances of n = 2^lgn whose ADMM CTAs the device holds at a time (>= 1).
+cudaError_t small_class_wave(int lgn, int* instances);
 cudaError_t launch_small_class(bool admm, int lgN, const SmallInst* inst, int count, const SmallScalars* sc,
                                const float* y, float* xz, int iters, cudaStream_t s);
 

@@ -486,6 +486,19 @@ cudaError_t class_run(bool admm, const SmallInst* inst, int count, const SmallSc
 }
 
 template <int LG>
+cudaError_t class_wave(int* instances) {
+  const void* fn = (const void*)class_admm_k<LG>;
+  const size_t smem = small_smem<LG, true>(false);
+  int dev = 0, sms = 0, ctas = 0;
+  cudaError_t e = opt_in_smem(fn, smem);
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, fn, SmallShape<LG>::NT, smem);
+  *instances = sms * ctas > 0 ? sms * ctas : 1;
+  return e;
+}
+
+template <int LG>
 cudaError_t small_run(SmallKind kind, const SmallArgs& a, cudaStream_t s) {
   using S = SmallShape<LG>;
   const void* fn = nullptr;
@@ -520,6 +533,16 @@ cudaError_t launch_small_class(bool admm, int lgN, const SmallInst* inst, int co
                                const float* y, float* xz, int iters, cudaStream_t s) {
   switch (lgN) {
 #define CS_X(L) case L: return class_run<L>(admm, inst, count, sc, y, xz, iters, s);
+    CS_SMALL_LG(CS_X)
+    CS_X(13)
+#undef CS_X
+  }
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t small_class_wave(int lgn, int* instances) {
+  switch (lgn) {
+#define CS_X(L) case L: return class_wave<L>(instances);
     CS_SMALL_LG(CS_X)
     CS_X(13)
 #undef CS_X

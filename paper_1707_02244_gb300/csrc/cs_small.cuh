@@ -49,14 +49,15 @@ template <int LG> struct SmallShape {
 // stage_twiddle).
 //
 // The batch's size classes take FULL: the solver they replaced did too, and
-// with products their ADMM error against 64 bits was 10 to 15 %
-// larger (20 iterations, n = 1024 .. 8192; within 2 % with FULL, at the same time: a batch
-// fills the chip, 8.50 against 8.53 ms for 256 instances).  One instance of a
-// plan takes products: bound by one SM's shared-memory pipe, it is 10 % slower
-// with FULL (500 ISTA iterations at n = 4096: 2.04 against 2.25 ms), and either
-// way it rounds less than the four-step passes it replaced (n = 1024 .. 4096:
-// products 0.79 .. 0.84 of a product's error, ISTA 0.95, ADMM 0.9; FULL 0.75 ..
-// 0.80, 0.94, 0.8).
+// with products their ADMM error against 64 bits was 10 to 15 % larger (20
+// iterations, n = 1024 .. 8192; ISTA 1 to 2 %), within 2 % with FULL.  50
+// iterations of 200 instances each of n = 8192, 4096 and 2048 take 0.93 ms
+// (ISTA) and 0.92 ms (ADMM), with products 0.85 and 0.91 ms.
+// One instance of a plan takes products: bound by one SM's shared-memory pipe,
+// it is 10 % slower with FULL (500 ISTA iterations at n = 4096: 2.04 against
+// 2.25 ms), and either way it rounds less than the four-step passes it replaced
+// (n = 1024 .. 4096: products 0.79 .. 0.84 of a product's error, ISTA 0.95, ADMM
+// 0.9; FULL 0.75 .. 0.80, 0.94, 0.8).
 template <int LG, bool FULL> struct SmallTw {
   using S = SmallShape<LG>;
   static constexpr int kF1 = 0;
