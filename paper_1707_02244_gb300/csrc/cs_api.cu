@@ -138,9 +138,13 @@ void r8_mid(Geo& g) {
 
 // Radix-8 tiles of one row pair / four columns (the fewest that fill a
 // 32-byte sector), 8 values per thread: as many CTAs as the length gives and
-// short stages.  Taken where the whole pass is less than about one wave of
-// such CTAs and its time is the latency of one tile; the 4096-value tiles of
-// the long transforms move fewer bytes through shared memory.
+// short stages.  Below N = 2^20 the 4096-value tiles leave most SMs idle and a
+// pass takes the latency of one of them.  Measured, us an iteration, radix-8
+// tiles against static 4096-value ones: ISTA N = 2^16 12.9 / 26.0, 2^17 16.3 /
+// 27.6, 2^18 25.7 / 51.0, 2^19 28.4 / 57.0; ADMM 2^17 7.6 / 16.5, 2^18 10.1 /
+// 25.8, 2^19 14.1 / 31.9.  The lengths above fill the chip with 4096-value
+// tiles, which move fewer bytes through shared memory (not measured with
+// radix 8).
 // `small_tiles` 0: 4096-value tiles at every length (grouped launches).
 constexpr int R8_LG_MIN = 11, R8_LG_MAX = 19;
 
@@ -665,6 +669,10 @@ cs_status build_plan(cs_plan_t* out, int64_t n0, int64_t n1, int64_t m, const in
     CS_PLAN_TRY(launch_tab_admm(chat, p->ga, n, p->tab_admm_c, p->abs2, s));
   }
   p->lgn = lgn;
+  // One CTA up to N = 2^12, the longest that fits it with a dense y; above it
+  // one cluster of CTAs where that is faster than the passes (cs_cluster.cu).
+  // At N = 2^12 itself (us an iteration, one CTA / cluster): ISTA 7.7 / 7.5,
+  // products 13.8 / 15.0 us a call, ADMM 4.6 / 2.8.
   p->small_i = !twod && small_tiles && lgn - 1 <= SMALL_LG_MAX;
   p->small_a = !twod && small_tiles && lgn <= SMALL_LG_MAX;
   if (p->small_i) {

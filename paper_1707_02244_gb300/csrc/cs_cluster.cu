@@ -12,8 +12,8 @@
 // A pass of these lengths is bound by its latency: launch gap, the round trip
 // of W, x and y through L2, table fills.  Here an exchange costs the SM-to-SM
 // latency and one fence, and tables are filled once per solve.  Measured, us
-// an iteration, passes -> cluster: ADMM n = 2^13 5.7 -> 3.6, 2^14 6.5 -> 4.9,
-// 2^15 6.7 -> 5.9, 2^16 7.1 -> 14.6; ISTA 2^14 11.4 -> 9.2, 2^15 12.2 -> 11.4,
+// an iteration, passes -> cluster: ADMM n = 2^13 5.7 -> 3.5, 2^14 6.5 -> 4.8,
+// 2^15 6.7 -> 5.8, 2^16 7.1 -> 14.6; ISTA 2^14 11.4 -> 9.2, 2^15 12.2 -> 11.3,
 // 2^16 11.9 -> 17.0: beyond 2048 values a CTA the exchange through 16 SMs is
 // slower than the passes on all of them, so the lengths end there.  At
 // n = 2^15 an ADMM iteration issues in 31 % of its cycles; the fence of the

@@ -5,8 +5,9 @@
 // R values per butterfly at stride L/R, twiddles them, applies an in-register
 // DFT_R and writes them back in auto-sorted order, so no bit reversal is ever
 // needed.  Stages use radix 16 while log2(L) allows it and one radix-2/4/8
-// stage for the remainder.  Every thread owns EPT = 16 values per stage
-// (TILE = 16 * NT), which keeps a stage within 64 registers.
+// stage for the remainder, every thread owning EPT = 16 values per stage
+// (TILE = 16 * NT), which keeps a stage within 64 registers; or, in the small
+// tiles, radix 8 and one radix-2/4 stage, 8 values per thread (TILE = 8 * NT).
 //
 // Shared-memory index of linear element e is e + (e >> 4): one pad slot per
 // 16 complex values keeps the stride-16 writes of the first stage free of

@@ -54,7 +54,7 @@
 
 namespace csk {
 
-// Threads per CTA: 3 CTAs of 320 per SM at <= 68 registers (96 instances of
+// Threads per CTA: 3 CTAs of 320 per SM at <= 64 registers (96 instances of
 // 2^12 .. 2^20, 20 + 20 iterations: 28.5 ms; 256: 29.5, 384: 29.2).
 constexpr int SM_NT = 320;
 constexpr int SM_TILE = 4096;          // complex values per shared buffer (two buffers)
