@@ -1398,14 +1398,28 @@ KParams kp_admm(const cs_plan_s* p, const CallArgs* ca, const float2* in, float2
 // iteration j's forward pair is transformed into wseg[j], where its mid pass
 // reads it and the reverse finds it, and its soft-threshold input is kept
 // (sseg[j]).
+//
+// For n = 2^18 .. 2^20 the passes stay on the exchange buffer instead and
+// wseg[j] is a copy of it: passes that go through a fresh buffer every iteration
+// were slower there by more than the copy takes.  Measured, us a gradient (T =
+// 75, K = 25; direct / copied): n = 2^16 2270 / 2332, 2^18 3245 / 3049, 2^19 3922
+// / 3884, 2^20 8397 / 7660, 2^21 10603 / 10879, 2^22 22747 / 23273.
 cudaError_t enqueue_admm_replay(cs_plan_s* p, int L, cudaStream_t s) {
   auto& G = p->ga_;
   const size_t n = (size_t)p->n;
-  cudaError_t e = launch_col(COL_ADMM_INIT, kp_admm(p, G.ca, p->W, G.wseg, nullptr), s);
+  const bool copy = p->lgn >= 18 && p->lgn <= 20;
+  // where iteration j's forward pair is transformed to, and kept
+  auto pair_at = [&](int j) { return copy || j >= L ? p->W : G.wseg + j * n; };
+  auto keep = [&](int j) {
+    return copy && j < L ? cudaMemcpyAsync(G.wseg + j * n, p->W, n * sizeof(float2), cudaMemcpyDeviceToDevice, s)
+                         : cudaSuccess;
+  };
+  cudaError_t e = launch_col(COL_ADMM_INIT, kp_admm(p, G.ca, p->W, pair_at(0), nullptr), s);
+  if (e == cudaSuccess) e = keep(0);
   for (int j = 0; j < L && e == cudaSuccess; ++j) {
-    e = launch_mid(MID_ADMM, kp_admm(p, G.ca + j, G.wseg + j * n, p->W, nullptr), s);
-    if (e == cudaSuccess)
-      e = launch_col(COL_ADMM_SEG, kp_admm(p, G.ca + j, p->W, j + 1 < L ? G.wseg + (j + 1) * n : p->W, nullptr), s);
+    e = launch_mid(MID_ADMM, kp_admm(p, G.ca + j, pair_at(j), p->W, nullptr), s);
+    if (e == cudaSuccess) e = launch_col(COL_ADMM_SEG, kp_admm(p, G.ca + j, p->W, pair_at(j + 1), nullptr), s);
+    if (e == cudaSuccess) e = keep(j + 1);
   }
   return e;
 }
