@@ -28,6 +28,8 @@
  *     latched in the plan and returned by cs_status_sync or by the next call
  *     that synchronises.
  *   - A plan is used from one host thread at a time and one stream.
+ *   - While the plan's stream is captured, cs_forward and cs_adjoint go into
+ *     the capture; cs_ista and cs_admm(_ex) do not (CS_ERR_CUDA).
  */
 #ifndef CS_H
 #define CS_H

@@ -398,6 +398,18 @@ cudaError_t run_chunk(cs_plan_s* p, SolveKind kind, int len, bool final_chunk, b
   return cudaGraphLaunch(it->second, p->stream);
 }
 
+// A solve does not go into a stream capture: the pass path launches graphs of
+// its own, and what a solve leaves out because the plan holds it already (B's
+// spectrum of the last rho, sigma) would be missing when the capture is
+// replayed after another solve.  The one-launch paths ask, as nothing else would
+// refuse them there.
+cudaError_t not_capturing(const cs_plan_s* p) {
+  if (!p->use_graphs) return cudaSuccess;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  const cudaError_t e = cudaStreamIsCapturing(p->stream, &st);
+  return e == cudaSuccess && st != cudaStreamCaptureStatusNone ? cudaErrorStreamCaptureUnsupported : e;
+}
+
 // Iterate up to the check points, every check_every iterations; with a monitor
 // tolerance, stop at the first one whose NMSE meets it.
 // step(done, len, final chunk, statistics) enqueues iterations done .. done +
@@ -876,6 +888,7 @@ cs_status cs_ista(cs_plan_t p, const float* y, float lambda, float tau, int iter
       !std::isfinite(lambda))
     return CS_ERR_ARG;
   cudaStream_t s = p->stream;
+  if (p->small_i || p->cluster_i) CS_TRY(not_capturing(p));
   if (stats) CS_TRY(cudaEventRecord(p->ev0, s));
   CallArgs a{};
   a.src = x;             // the prologue transforms x(0) in natural order
@@ -958,6 +971,7 @@ namespace {
 cs_status admm_impl(cs_plan_t p, const float* y, float lambda, const cs_admm_params* prm, int iters, int warm,
                     float* x, float* z, float* mu, float* nu, float* v, cs_stats* stats) {
   cudaStream_t s = p->stream;
+  if (p->small_a || p->cluster_a) CS_TRY(not_capturing(p));
   if (stats) CS_TRY(cudaEventRecord(p->ev0, s));
   const size_t nb = p->n * sizeof(float);
   p->launches = 0;

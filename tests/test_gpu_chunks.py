@@ -35,6 +35,43 @@ def _plan(cs, n, seed):
     return plan, c, rows, x, y, f32(0.9 / np.max(np.abs(chat) ** 2))
 
 
+@pytest.mark.parametrize("n", [1024, 1 << 13, 1 << 14])
+def test_solves_do_not_go_into_a_capture(cs, n):
+    """A captured solve would leave out what the plan held at that moment (the
+    spectrum of B for its rho), and answer wrongly when it is replayed after
+    another one.  Refused as on the pass path; products are captured."""
+    torch, dev = torch_dev()
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        plan, c, rows, _, y, tau = _plan(cs, n, 8150 + n)
+        yd, x, z, p = to_dev(y), torch.zeros(n, device=dev), torch.empty(n, device=dev), torch.empty(plan.m, device=dev)
+        try:
+            cs.cs_admm(plan, yd, 1e-3, 1.0, 3, z, stats=False)
+            cs.cs_forward(plan, z, p)
+            st.synchronize()
+            want_z, want_p = z.clone(), p.clone()
+            for solve in (lambda: cs.cs_ista(plan, yd, 1e-3, tau, 3, x, stats=False),
+                          lambda: cs.cs_admm(plan, yd, 1e-3, 2.0, 3, z, stats=False)):
+                with torch.cuda.graph(torch.cuda.CUDAGraph(), stream=st):
+                    p.zero_()
+                    with pytest.raises(cs.CsError) as err:
+                        solve()
+                assert err.value.code == 3   # CS_ERR_CUDA
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=st):
+                cs.cs_forward(plan, z, p)
+            cs.cs_admm(plan, yd, 1e-3, 2.0, 3, z, stats=False)
+            zo = O.admm_fft(c, rows, y.astype(np.float64), f32(1e-3), sigma=2.0, rho=2.0, iters=3)["z"]
+            st.synchronize()
+            assert rel_l2(host(z), zo) <= 1e-5
+            cs.cs_admm(plan, yd, 1e-3, 1.0, 3, z, stats=False)
+            g.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(z, want_z) and torch.equal(p, want_p)
+        finally:
+            plan.close()
+
+
 @pytest.mark.parametrize("n", [64, 4096, 1 << 13, 1 << 15, 1 << 17])
 def test_profile_pass_inputs(cs, n):
     """The pass kernels that the measurement hook launches find inputs laid out:
